@@ -29,6 +29,17 @@ int ffbs_wide_wpc(int L) {
     }
 }
 
+// units that a CTA of the FP32 streaming kernel filters before it draws their worldlines
+int ffbs_wide_batch(int L) {
+    switch (L) {
+#define HQMC_CASE(n) \
+    case n: return WideGeo<float, n>::NB;
+        HQMC_WIDE_SIZES(HQMC_CASE)
+#undef HQMC_CASE
+        default: return 1;
+    }
+}
+
 // both Gaussian flags get their limits; the grid follows the smaller residency
 cudaError_t ffbs_wide_occupancy(int L, bool fp64, int *blocks) {
     cudaError_t e = wide_occ_dispatch<false>(L, fp64, blocks);

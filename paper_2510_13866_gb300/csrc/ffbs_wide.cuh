@@ -20,16 +20,25 @@
 // partials, so results do not depend on scheduling.
 //
 // f_l = W_l . alpha_l is streamed to the worldline's slot in 16-byte chunks (chunk j of
-// line p at j*L + p, coalesced over the lines); the backward pass prefetches each slice
-// into shared memory with cp.async and samples x_l ~ max(f_l(y), 0) G(x_{l+1} - y) by the
-// row-major inverse CDF, one row per thread.
+// line p at j*L + p, coalesced over the lines).  The backward pass samples
+// x_l ~ max(f_l(y), 0) G(x_{l+1} - y) by the row-major inverse CDF: FP32 Hirsch chains with
+// short-ranged G (ChainDev.win_R) draw from a window around the worldline, one warp per
+// worldline (ffbs_window.cuh); the others prefetch each whole slice into shared memory with
+// cp.async, one row per thread.
 #pragma once
 
 #include <cuda_bf16.h>
 
 #include "ffbs.cuh"
+#include "ffbs_window.cuh"
 
 namespace hqmc {
+
+// Units (groups of WPC worldlines) that one CTA of the FP32 streaming kernel filters before it
+// draws their worldlines, a warp each: as many as give every warp a worldline or two.  Drawn one
+// unit at a time, one warp (two at L = 48) worked and the CTA's others waited.
+template <int L>
+constexpr int kWideBatch = L == 48 ? 3 : L / 32;
 
 template <typename T, int L>
 struct WideGeo {
@@ -43,18 +52,23 @@ struct WideGeo {
     static constexpr size_t XTR = size_t(L) * LP * sizeof(T);
     static constexpr size_t XPF = size_t(L / CH) * (L + 1) * 16;
     static constexpr size_t XB = a16(XTR > XPF ? XTR : XPF);
+    // FP32 streaming: units whose worldlines are drawn together after their forward passes
+    // (kWideBatch), and one window ring per warp in the place of the transpose buffers
+    static constexpr int NB = sizeof(T) == 4 ? kWideBatch<L> : 1;
+    static constexpr size_t XALL = sizeof(T) == 4 && NW * kWinBytes > WPC * XB ? NW * kWinBytes : WPC * XB;
     static constexpr size_t MIXB = a16(size_t(2 * L) * sizeof(T));  // (al, -al, be, -be) per k
-    static constexpr size_t G2B = a16(size_t(2 * L) * sizeof(T));
+    static constexpr size_t G2B = a16(size_t(2 * L) * sizeof(T));  // per unit of a batch
     static constexpr size_t WXB = a16(size_t(WPC) * L * sizeof(T));
-    static constexpr size_t HLB = a16(size_t(L) * sizeof(float));
+    static constexpr size_t HLB = a16(size_t(L) * sizeof(float));  // per unit of a batch
+    static constexpr size_t UNB = a16(NB * sizeof(WinUnit));
     static constexpr size_t REDB = a16(size_t(2 * NW * WPC + 4 * WPC) * sizeof(T));
     static constexpr size_t IB = 64;  // work unit, crossings, fallbacks, end exponents
     static constexpr size_t UB = a16(size_t(WPC) * 8);
-    static constexpr size_t BYTES = WPC * XB + MIXB + G2B + WXB + HLB + REDB + IB + UB;
+    static constexpr size_t BYTES = XALL + MIXB + NB * (G2B + HLB) + WXB + REDB + IB + UB + UNB;
     // resident CTAs per SM the register budget is sized for
     static constexpr int MINB = sizeof(T) == 4 ? (L == 128 ? 2 : L == 64 ? 8 : 6) : (L == 128 ? 1 : 2);
     static_assert(L % 4 == 0 && NT % 32 == 0 && NT <= 256, "wide geometry");
-    static_assert(XB >= XPF, "prefetch buffer");
+    static_assert(XB >= XPF && WPC <= 2, "prefetch buffer");
 };
 
 // 16-byte moves between a register array (elements k .. k + 16/sizeof(T) - 1, constant k
@@ -167,15 +181,15 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *sp = smem_raw;
     T *xbuf_all = reinterpret_cast<T *>(sp);
-    sp += WPC * G::XB;
+    sp += G::XALL;
     T *mix = reinterpret_cast<T *>(sp);
     sp += G::MIXB;
-    T *g2 = reinterpret_cast<T *>(sp);
-    sp += G::G2B;
+    T *g2_all = reinterpret_cast<T *>(sp);
+    sp += G::NB * G::G2B;
     T *wx_all = reinterpret_cast<T *>(sp);
     sp += G::WXB;
-    float *hl = reinterpret_cast<float *>(sp);
-    sp += G::HLB;
+    float *hl_all = reinterpret_cast<float *>(sp);
+    sp += G::NB * G::HLB;
     T *wred = reinterpret_cast<T *>(sp);  // [NW][WPC] sums, [NW][WPC] maxima, [WPC] x 4 end values
     T *wmx = wred + NW * WPC;
     T *endv = wmx + NW * WPC;             // [WPC] end value, [WPC] top, [WPC] spare
@@ -183,6 +197,8 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
     int *ibuf = reinterpret_cast<int *>(sp);  // [0] unit, [1 + w] crossing, [5 + w] fallback, [9 + w] esum
     sp += G::IB;
     uint64_t *ubuf = reinterpret_cast<uint64_t *>(sp);  // [WPC] uniforms of the slice
+    sp += G::UB;
+    WinUnit *units = reinterpret_cast<WinUnit *>(sp);  // filtered units to be drawn
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int w = tid % WPC;  // worldline of the CTA
@@ -190,8 +206,26 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
     T *xb = reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(xbuf_all) + w * G::XB);
     T *wx = wx_all + w * L;
     const uint64_t sweep = *st.sweep;
-    T *slot = reinterpret_cast<T *>(fl.scratch) + (long long)blockIdx.x * fl.slot_elems +
-              (long long)w * (fl.slot_elems / WPC);
+    constexpr bool WIN = sizeof(T) == 4 && !CKPT && !GAUSS;
+    // fl.batch slots per CTA: one for each unit that waits to be drawn
+    T *slot0 = reinterpret_cast<T *>(fl.scratch) + (long long)blockIdx.x * fl.batch * fl.slot_elems;
+    int nwait = 0;
+    // draws the waiting units, a warp per worldline
+    auto draw_waiting = [&]() {
+        if constexpr (WIN) {
+            __syncthreads();
+            unsigned char *ring = smem_raw + warp * kWinBytes;
+#pragma unroll 1
+            for (int k = warp; k < nwait * WPC; k += NW) {
+                const int u = k / WPC, ww = k % WPC;
+                if (ww >= units[u].nwl) continue;
+                win_backward<L, WPC>(st, units[u], ww,
+                                     slot0 + (long long)u * fl.slot_elems + (long long)ww * (fl.slot_elems / WPC),
+                                     g2_all + u * (G::G2B / sizeof(T)), hl_all + u * (G::HLB / sizeof(float)), ring, sweep, lane);
+            }
+        }
+        nwait = 0;
+    };
 
     // per-worldline sum and maximum over the CTA (fixed order: deterministic)
     auto wl_sum = [&](T v) -> T {
@@ -210,7 +244,13 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
         if (tid == 0) ibuf[0] = int(atomicAdd(fl.next_unit, 1u));
         __syncthreads();
         const long long q = ibuf[0];
-        if (q >= fl.total_units) break;
+        if (q >= fl.total_units) {
+            if (WIN && nwait > 0) draw_waiting();
+            break;
+        }
+        T *slot = slot0 + (long long)nwait * fl.slot_elems + (long long)w * (fl.slot_elems / WPC);
+        T *g2 = g2_all + nwait * (G::G2B / sizeof(T));
+        float *hl = hl_all + nwait * (G::HLB / sizeof(float));
         int lo = 0, hi = fl.nclass - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -277,6 +317,7 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
             for (int r = 0; r < L; ++r) v[r] = (has && p == sy && r == sx) ? wv : T(0);
         }
         int esum = 0;
+        bool normal = true;  // every slice's sum was in range, so the stored f are normalised
         // the slice of block position i (positions run from the block start l0)
         auto slice_of = [&](int i) {
             int s_ = l0 + i;
@@ -321,7 +362,10 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
         auto renorm_w = [&](int i, T s, bool count) -> int {
             int e = 0;
             if (s > T(0) && s < T(1e30)) e = fbits<T>::exponent(s);
-            else if (count && has && p == 0) atomicAdd(&st.meas[c].degenerate, 1ull);
+            else {
+                normal = false;
+                if (count && has && p == 0) atomicAdd(&st.meas[c].degenerate, 1ull);
+            }
             const T sc = fbits<T>::pow2(-e);
             const int l1 = slice_of(i + 1);
             // the new layout is C (lines = x) when i is even: the field by columns
@@ -468,6 +512,24 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
         if (!(GAUSS && cd.gauss)) book();
 
         // ---- backward sampling ----
+        if constexpr (WIN) {
+            if (cd.win_R > 0) {
+                WinUnit &un = units[nwait];
+                if (tid == 0) {
+                    un.c = c;
+                    un.sg = sg;
+                    un.pw0 = pw0;
+                    un.nwl = nwl;
+                    un.l0 = l0;
+                    un.len = len;
+                    un.le = le;
+                    un.wi = wi;
+                }
+                if (p == 0) un.normal[w] = normal ? 1 : 0;
+                if (++nwait == fl.batch) draw_waiting();
+                continue;
+            }
+        }
         // slice i of the slots -> xbuf: R slices (i even) chunk for chunk, C slices (i odd)
         // into rows of pitch L+1 chunks so that the row-wise reads below are conflict-free
         // f of position i: the streamed slice, or with checkpoints the recomputed segment

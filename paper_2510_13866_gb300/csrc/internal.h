@@ -10,6 +10,7 @@ namespace hqmc {
 
 constexpr int kMaxL = 128;
 constexpr int kPTab = 64;  // P(s=+1 | m) tabulated for |m| <= kPTab, computed beyond
+constexpr int kWinHalf = 12;  // half width of the backward draw's window (ffbs_window.cuh)
 
 // Per-chain tables, computed on the host in FP64 at set_params.
 struct ChainTab {
@@ -54,6 +55,10 @@ struct ChainDev {
     long long v_off;    // element offset of [2][M][N] gradient arrays
     long long meas_off; // offset into the measurement arrays (N per chain)
     long long perm_off; // int offset of the permutation P [2][Nsig] then its inverse [2][Nsig]
+    // windowed backward draw (FP32, Hirsch fields): steps beyond which G is negligible (0: no
+    // window) and the least conditional total S the window answers for (window_rule)
+    int win_R;
+    float win_min;
 };
 
 // Per-chain measurement accumulators (device, zeroed at reset).
@@ -133,6 +138,7 @@ struct FfbsLaunch {
     int ckpt_bf16;
     long long seg_off;
     int gauss;                 // some chain of the class has a Gaussian field (U < 0)
+    int batch;                 // wide kernel: slots per CTA (units filtered before they are drawn)
 };
 
 // One launch of the adjoint kernel covers the chains of one lattice size.
@@ -168,6 +174,7 @@ cudaError_t launch_slice(const DevState &st, int nchains, int max_M, int max_L, 
                          bool measure, cudaStream_t stream);
 cudaError_t configure_slice(int max_L, int S);
 int slice_group(int max_L, int requested, long long work_slices, int num_sms);
+void window_rule(const ChainTab &tb, int L, double wmax, ChainDev &d);
 void host_chain_table(int L, double t, double U, double dtau, ChainTab &tb, double *lam);
 cudaError_t launch_advance(const DevState &st, cudaStream_t stream);
 // local link updates: the largest (worldline, slice) count of one colour of a chain, and

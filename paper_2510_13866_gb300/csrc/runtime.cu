@@ -34,6 +34,7 @@ cudaError_t grad_wide_occupancy(int L, bool fp64, int *blocks);
 cudaError_t ffbs_wide_occupancy(int L, bool fp64, int *blocks);
 bool ffbs_wide_supported(int L);
 int ffbs_wide_wpc(int L);
+int ffbs_wide_batch(int L);
 
 // register-line sizes (one warp-group per pair) and wide sizes (one thread per line of
 // each worldline, one or two worldlines per CTA); both precisions
@@ -60,6 +61,9 @@ struct HostChain {
     bool set = false;
 };
 
+// Scratch of a wide FP32 class up to which its CTAs take several slots each: 5% of the device
+constexpr size_t kBatchBytes = size_t(14) << 30;
+
 struct LClass {
     int L = 0;
     std::vector<int> chains;
@@ -78,6 +82,7 @@ struct LClass {
     // seg_off of a worldline's slot of wl_elems floats (ckpt_K = 0: every f streamed)
     int ckpt_K = 0;
     long long seg_off = 0, wl_elems = 0;
+    int batch = 1;         // slots per CTA of a wide FP32 streaming class
     // FFBS slot per group, in the kernel's elements (pairs for L <= 32, scalars of the CTA's
     // worldlines for wide): the f storage of each worldline, then len_max per-position maxima
     // of the forward messages (Gaussian-field units), padded to whole 16-byte chunks
@@ -140,6 +145,8 @@ struct hqmc_ctx {
     std::vector<unsigned> keep_parity;
     unsigned long long keep_sweep = 0;
     bool keep_started = false;
+
+    bool batch_units = true;  // several slots per CTA of the wide classes (off where memory is short)
 
     // adjoint: checkpoint stride (0 = ceil(sqrt M)) and format, context-owned scratch
     int ckpt_stride = 0;
@@ -250,6 +257,27 @@ double hirsch_lambda(double U, double dtau) { return std::acosh(std::exp(0.5 * d
 }  // namespace
 
 namespace hqmc {
+// Window of the backward draw (ffbs_window.cuh).  WinR is the least R with g(R + 1) <= 2^-60 g(0):
+// the sites beyond it then hold less than 2^-36 of any total S >= win_min = 2^36 4 g(R + 1) g(0)
+// max W, and win_min stays below 2^-22 of the largest weight, so that almost every draw is
+// answered (t dtau = 1/32, 0.05, 0.1: R = 8, 9, 10).  Hops that need R > kWinHalf - 1 (t dtau
+// above 0.14) leave no margin for the moves between load and draw: no window.
+void window_rule(const ChainTab &tb, int L, double wmax, ChainDev &d) {
+    d.win_R = 0;
+    d.win_min = 0.f;
+    if (L <= 2 * kWinHalf + 1) return;
+    double far = 0.0;  // the largest g beyond R
+    for (int R = L / 2 - 1; R >= 1; --R) {
+        far = std::max(far, tb.g_d[R + 1]);
+        if (far > 0x1.0p-60 * tb.g_d[0]) return;
+        if (R > kWinHalf - 1) continue;
+        const double m = 0x1.0p+36 * 4.0 * far * tb.g_d[0] * wmax;
+        if (!(m < 1e30)) return;
+        d.win_R = R;
+        d.win_min = float(std::max(m, 1e-30));
+    }
+}
+
 // Tables and lambda of one chain, for entry points that do not own a context.
 void host_chain_table(int L, double t, double U, double dtau, ChainTab &tb, double *lam) {
     HostChain h;
@@ -494,6 +522,14 @@ int plan_layout(hqmc_ctx *c, size_t *total) {
         k.slot_elems = (per_wl + aux) * (is_big(k.L) ? ffbs_wide_wpc(k.L) : 1);
         const size_t elem = is_big(k.L) ? (f64 ? 8 : 4) : (f64 ? 16 : 8);
         k.scratch_bytes = size_t(k.groups) * size_t(k.slot_elems) * elem;
+        // wide FP32 classes that stream f: more slots per CTA, so that several units are drawn
+        // at once, while the class stays within kBatchBytes and every CTA has the units
+        k.batch = 1;
+        if (is_big(k.L) && !f64 && k.ckpt_K == 0 && c->batch_units) {
+            const long long most = std::min<long long>(kBatchBytes / k.scratch_bytes, (k.total_units + k.grid - 1) / k.grid);
+            k.batch = int(std::max(1LL, std::min<long long>(ffbs_wide_batch(k.L), most)));
+            k.scratch_bytes *= k.batch;
+        }
         k.scratch_off = take(k.scratch_bytes);
     }
     *total = round_up(off, 256);
@@ -528,12 +564,22 @@ P rebase(P p, unsigned char *base) {
     return reinterpret_cast<P>(base + reinterpret_cast<size_t>(p));
 }
 
+// plan_layout within `limit` bytes: without the wide classes' extra slots where the layout with
+// them is larger.
+int plan_within(hqmc_ctx *c, size_t limit, size_t *need) {
+    c->batch_units = true;
+    int rc = plan_layout(c, need);
+    if (rc || *need <= limit) return rc;
+    c->batch_units = false;
+    return plan_layout(c, need);
+}
+
 // Plan, bind memory (attached or owned), upload tables and initialise the state.
 int prepare(hqmc_ctx *c) {
     if (c->ready) return HQMC_OK;
     HQMC_CUDA(c, cudaSetDevice(c->device));
     size_t need = 0;
-    int rc = plan_layout(c, &need);
+    int rc = plan_within(c, c->attached ? c->attached_bytes : SIZE_MAX, &need);
     if (rc) return rc;
     if (c->attached) {
         if (c->attached_bytes < need) return fail(c, HQMC_ERR_NOMEM, "attached workspace too small");
@@ -542,6 +588,12 @@ int prepare(hqmc_ctx *c) {
     } else {
         void *p = nullptr;
         cudaError_t e = cudaMalloc(&p, need);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            rc = plan_within(c, 0, &need);
+            if (rc) return rc;
+            e = cudaMalloc(&p, need);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(c, HQMC_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -578,7 +630,10 @@ int prepare(hqmc_ctx *c) {
     cudaStream_t st = c->stream;
     HQMC_CUDA(c, cudaMemsetAsync(c->base, 0, need, st));
     std::vector<ChainTab> tabs(c->nchains);
-    for (int i = 0; i < c->nchains; ++i) build_tab(c->ch[i], tabs[i], c->cdev[i].lam);
+    for (int i = 0; i < c->nchains; ++i) {
+        build_tab(c->ch[i], tabs[i], c->cdev[i].lam);
+        window_rule(tabs[i], c->ch[i].L, std::exp(c->cdev[i].lam), c->cdev[i]);
+    }
     HQMC_CUDA(c, cudaMemcpyAsync((void *)s.chains, c->cdev.data(), sizeof(ChainDev) * c->nchains, cudaMemcpyHostToDevice, st));
     HQMC_CUDA(c, cudaMemcpyAsync((void *)s.tabs, tabs.data(), sizeof(ChainTab) * c->nchains, cudaMemcpyHostToDevice, st));
     for (auto &k : c->classes) {
@@ -731,6 +786,7 @@ int enqueue_sweep(hqmc_ctx *c, cudaStream_t st, bool capture) {
         fl.ckpt_K = cl.ckpt_K;
         fl.ckpt_bf16 = c->fstore == HQMC_FSTORE_BF16 ? 1 : 0;
         fl.seg_off = cl.seg_off;
+        fl.batch = cl.batch;
         cudaStream_t s = k == 0 ? st : c->aux[k - 1];
         HQMC_CUDA(c, cudaMemsetAsync(fl.next_unit, 0, sizeof(unsigned), s));
         const int wpc = default_wpc(c, cl.L);
@@ -892,6 +948,7 @@ int hqmc_set_params(hqmc_ctx *c, int chain, double t, double U, double beta, dou
             d.gcoup = std::sqrt(std::fabs(c->ch[i].U) * c->ch[i].dtau);
             ChainTab tb;
             build_tab(c->ch[i], tb, d.lam);
+            window_rule(tb, c->ch[i].L, std::exp(d.lam), d);
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.chains + i), &d, sizeof(ChainDev), cudaMemcpyHostToDevice, c->stream));
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.tabs + i), &tb, sizeof(ChainTab), cudaMemcpyHostToDevice, c->stream));
             if (d.gauss) {
@@ -1148,11 +1205,18 @@ int hqmc_workspace_size(hqmc_ctx *c, size_t *bytes) {
     DevState keep = c->st;
     auto keep_cdev = c->cdev;
     auto keep_cls = c->classes;
-    int rc = plan_layout(c, &need);
+    const bool keep_batch = c->batch_units;
+    // a workspace for the wide classes' extra slots is asked for only where the device has the
+    // room for it (or what is attached already holds it)
+    size_t room = 0, total = 0;
+    HQMC_CUDA(c, cudaSetDevice(c->device));
+    HQMC_CUDA(c, cudaMemGetInfo(&room, &total));
+    int rc = plan_within(c, std::max(room, c->attached_bytes), &need);
     if (c->ready) {
         c->st = keep;
         c->cdev = keep_cdev;
         c->classes = keep_cls;
+        c->batch_units = keep_batch;
     }
     if (rc) return rc;
     *bytes = need;
@@ -1166,7 +1230,7 @@ int hqmc_attach_workspace(hqmc_ctx *c, void *dev_ptr, size_t bytes) {
     c->attached = static_cast<unsigned char *>(dev_ptr);
     c->attached_bytes = bytes;
     size_t need = 0;
-    int rc = plan_layout(c, &need);
+    int rc = plan_within(c, bytes, &need);
     if (rc) return rc;
     if (bytes < need) {
         c->attached = nullptr;
