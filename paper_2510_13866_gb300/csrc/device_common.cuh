@@ -352,10 +352,8 @@ __device__ __forceinline__ void fft(cvec<V> (&a)[N]) {
     }
 }
 
-// Building blocks of conv_line with the spectrum exposed, for passes that apply more
-// than one line kernel to the same line (the adjoint applies g and dg/dt):
+// Building blocks of conv_line:
 //   line_fwd: spectrum of the line (even L: DFT_n of the packed line, odd L: DFT_L)
-//   spec_mix: out = mix(in), or out += mix(in) with ACC (out must not alias in)
 //   line_inv: the line whose spectrum is z (the 1/n or 1/L factor is in the mix)
 template <int L>
 struct line_spec {
@@ -386,31 +384,6 @@ __device__ __forceinline__ void line_inv(cvec<V> (&z)[line_spec<L>::K], V (&v)[L
     } else {
 #pragma unroll
         for (int m = 0; m < L; ++m) v[m] = z[m].re;
-    }
-}
-
-template <int L, bool ACC, typename V>
-__device__ __forceinline__ void spec_mix(cvec<V> (&out)[line_spec<L>::K], const cvec<V> (&in)[line_spec<L>::K],
-                                         const V *mix) {
-    if constexpr (L % 2 == 0) {
-        constexpr int n = L / 2;
-        static_for<0, n>([&](auto KI) {
-            constexpr int k = decltype(KI)::value;
-            constexpr int kp = (n - k) % n;
-            V al, be;
-            load_mix(mix, k, al, be);
-            const V re = vfma(in[k].re, al, vmul(in[kp].im, be));
-            const V im = vfma(in[k].im, al, vmul(in[kp].re, be));
-            if constexpr (ACC) out[k] = {vadd(out[k].re, re), vadd(out[k].im, im)};
-            else out[k] = {re, im};
-        });
-    } else {
-#pragma unroll
-        for (int k = 0; k < L; ++k) {
-            const V w = load_mix1(mix, k);
-            if constexpr (ACC) out[k] = {vfma(in[k].re, w, out[k].re), vfma(in[k].im, w, out[k].im)};
-            else out[k] = {vmul(in[k].re, w), vmul(in[k].im, w)};
-        }
     }
 }
 

@@ -16,10 +16,16 @@
 // in BF16 with the slice's power-of-two exponent (FP32 context) or in the context's own
 // precision; the reverse pass recomputes each K-slice segment into a per-group buffer
 // (L2-resident) and walks it backwards.  One group of lanes owns a pair of same-spin
-// worldlines, as in the FFBS kernel; dG/dt * b shares the line spectra of G * b:
-//   x lines:  Z = DFT(b);  A = IDFT(mix_g Z),  Ad = IDFT(mix_dg Z)      (one transpose each)
-//   y lines:  ZA = DFT(A), ZAd = DFT(Ad);  H = IDFT(mix_g ZA),
-//             D = IDFT(mix_g ZAd + mix_dg ZA)                       (= dG/dt * b)
+// worldlines, as in the FFBS kernel.
+//
+// The t-derivative needs no transform of its own.  G = exp(t dtau A) with A = A_x + A_y the
+// lattice adjacency, so dG/dt = dtau (A_x + A_y) G, and A commutes with G:
+//     <F_l, (dG/dt) * b_{l+1}> = dtau (<F_l, A_r H_l> + <A_c alpha_{l+1}, b_{l+1}>),
+// where r is the direction that slice l's layout keeps in registers and c the other one, which
+// slice l + 1's layout keeps in registers: both sums are over neighbours in a lane's own line.
+// Carrying (dG/dt) * b as a second message took 7 half-length FFTs and two transposes per reverse
+// slice instead of 4 and one.  The kernel is bound by the FMA pipe: L = 16, M = 80, 128 chains with a
+// given v, 2.87 ms before this and exp_table_kernel, 2.17 ms with both (and 35 us for the table).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -34,15 +40,8 @@ struct GradGeo {
     using V = vec2_t<T>;
     static constexpr size_t XBUF = F::XBUF;
     static constexpr size_t MIXB = F::MIXB;
-    static constexpr size_t GROUP_BYTES = XBUF + 2 * MIXB;
+    static constexpr size_t GROUP_BYTES = XBUF + MIXB;
 };
-
-template <typename T>
-__device__ __forceinline__ const T *tab_mixd(const ChainTab &tb);
-template <>
-__device__ __forceinline__ const float *tab_mixd<float>(const ChainTab &tb) { return tb.mixd_f; }
-template <>
-__device__ __forceinline__ const double *tab_mixd<double>(const ChainTab &tb) { return tb.mixd_d; }
 
 template <typename T>
 __device__ __forceinline__ T exp_t(T x);
@@ -65,7 +64,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
     using FG = FfbsGeo<T, L>;
     using V = vec2_t<T>;
     constexpr int N = L * L;
-    constexpr int GW = FG::GW, LP = FG::LP, CH = FG::CH, KS = line_spec<L>::K;
+    constexpr int GW = FG::GW, LP = FG::LP, CH = FG::CH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -76,7 +75,6 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
     unsigned char *gsm = smem_raw + size_t(warp * FG::GPW + gw) * G::GROUP_BYTES;
     V *xbuf = reinterpret_cast<V *>(gsm);
     V *mixg = reinterpret_cast<V *>(gsm + G::XBUF);
-    V *mixdg = reinterpret_cast<V *>(gsm + G::XBUF + G::MIXB);
     const long long gid = ((long long)blockIdx.x * wpc + warp) * FG::GPW + gw;
     const long long ngroups = (long long)gridDim.x * wpc * FG::GPW;
     unsigned char *ck = reinterpret_cast<unsigned char *>(gk.ckpt) + gid * gk.ckpt_bytes;
@@ -125,6 +123,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         const uint32_t *srow = st.sbits + cd.s_off;
         const uint32_t *scol = srow + (long long)M * L * cd.wpl;
         const T *vlog = vlog_all ? vlog_all + cd.v_off + (long long)sg * M * N : nullptr;
+        const T *wtab = gk.w ? static_cast<const T *>(gk.w) + cd.w_off + (long long)sg * M * N : nullptr;
         T *dvp = dv_all ? dv_all + cd.v_off + (long long)sg * M * N : nullptr;
         // vector reductions need every slice's row start 16-byte aligned
         const bool dv_v4 = dvp && (N % 4 == 0) && (reinterpret_cast<uintptr_t>(dvp) & 15) == 0;
@@ -134,11 +133,8 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
 
         __syncwarp(gmask);
         {
-            const T *src = tab_mix<T>(tb), *srcd = tab_mixd<T>(tb);
-            for (int j = gl; j < L; j += GW) {
-                mixg[j] = vsplat(src[j]);
-                mixdg[j] = vsplat(srcd[j]);
-            }
+            const T *src = tab_mix<T>(tb);
+            for (int j = gl; j < L; j += GW) mixg[j] = vsplat(src[j]);
         }
         __syncwarp(gmask);
 
@@ -147,7 +143,9 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         // v <- v . W_l . (s0, s1)  (slice l's layout)
         auto mul_w = [&](V (&v)[L], int l, T s0, T s1) {
             if (!active) return;
-            if (vlog) {
+            if (wtab) {
+                mul_gauss_line<T, L>(v, wtab + (long long)l * N + gl * L, s0, s1);
+            } else if (vlog) {
                 const T *vl = vlog + (long long)l * N;
 #pragma unroll
                 for (int r = 0; r < L; ++r) {
@@ -162,6 +160,36 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                 const V A = {wp * s0, wp * s1}, B = {wm * s0, wm * s1};
 #pragma unroll
                 for (int r = 0; r < L; ++r) v[r] = vmul(v[r], ((w >> r) & 1u) ? A : B);
+            }
+        };
+        // W_l along this lane's line (1 in idle lanes)
+        auto line_w = [&](int l, T (&w)[L]) {
+            const T *line = wtab ? wtab + (long long)l * N + gl * L
+                                 : (!vlog && cd.gauss) ? gauss_line<T>(st, cd, (l & 1) != 0, l, gl) : nullptr;
+            if (!active) {
+#pragma unroll
+                for (int r = 0; r < L; ++r) w[r] = T(1);
+            } else if (line) {
+                if constexpr (sizeof(T) == 4 && L % 4 == 0) {
+#pragma unroll
+                    for (int j = 0; j < L / 4; ++j) {
+                        const float4 q = reinterpret_cast<const float4 *>(line)[j];
+                        w[4 * j] = q.x;
+                        w[4 * j + 1] = q.y;
+                        w[4 * j + 2] = q.z;
+                        w[4 * j + 3] = q.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < L; ++r) w[r] = line[r];
+                }
+            } else if (vlog) {
+#pragma unroll
+                for (int r = 0; r < L; ++r) w[r] = exp_t<T>(vlog[(long long)l * N + site(l, r)]);
+            } else {
+                const uint32_t bits = ((l & 1) ? scol : srow)[((long long)l * L + gl) * cd.wpl];
+#pragma unroll
+                for (int r = 0; r < L; ++r) w[r] = ((bits >> r) & 1u) ? wp : wm;
             }
         };
         auto sums = [&](const V (&v)[L], T &s0, T &s1) {
@@ -233,6 +261,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         mul_w(f, 0, T(1), T(1));
         int esum0 = 0, esum1 = 0;
         T fin0 = T(1), fin1 = T(1);
+        T nb0 = T(0), nb1 = T(0);  // alpha_M at the two neighbours of x0 along the last layout's lines
         for (int l = 0; l < M; ++l) {
             if (l % K == 0) ck_store(l / K, f, esum0, esum1);
             conv2(f);
@@ -252,6 +281,10 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                 const T c1 = reg_select<L>(f, reg1).y;
                 fin0 = __shfl_sync(gmask, c0, own0, GW);
                 fin1 = __shfl_sync(gmask, c1, own1, GW);
+                const int up0 = reg0 + 1 == L ? 0 : reg0 + 1, dn0 = reg0 == 0 ? L - 1 : reg0 - 1;
+                const int up1 = reg1 + 1 == L ? 0 : reg1 + 1, dn1 = reg1 == 0 ? L - 1 : reg1 - 1;
+                nb0 = __shfl_sync(gmask, reg_select<L>(f, up0).x + reg_select<L>(f, dn0).x, own0, GW);
+                nb1 = __shfl_sync(gmask, reg_select<L>(f, up1).y + reg_select<L>(f, dn1).y, own1, GW);
             }
         }
         if (gl == 0) {
@@ -276,9 +309,9 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                 b[r].y = (bC ? (gl == ax1 && r == ay1) : (gl == ay1 && r == ax1)) ? T(1) : T(0);
             }
         }
-        // d log Z / dt: per-slice ratios in the context precision, compensated (Kahan) sums
+        // d log Z / dt over dtau: per-slice ratios in the context precision, compensated (Kahan) sums
         // (no FP64 instruction per slice in the FP32 context)
-        T dts0 = T(0), dtc0 = T(0), dts1 = T(0), dtc1 = T(0);
+        T dts0 = nb0 / fin0, dtc0 = T(0), dts1 = nb1 / fin1, dtc1 = T(0);
         auto kahan = [](T &sum, T &comp, T v) {
             const T y = v - comp;
             const T t = sum + y;
@@ -288,67 +321,63 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         const int nseg = (M + K - 1) / K;
         for (int s = nseg - 1; s >= 0; --s) {
             const int lb = s * K, le = min(M, lb + K);
-            // recompute F_lb .. F_{le-1} into the segment buffer (same lane, same slots)
-            ck_load(s, f);
-            for (int l = lb; l < le; ++l) {
+            // recompute the segment (same lane, same slots): F_lb from its checkpoint, then
+            // alpha_{lb+1} .. alpha_{le-1}, normalised
+            auto put = [&](int l) {
                 if (active) {
                     V *dst = seg + (long long)(l - lb) * N;
 #pragma unroll
                     for (int r = 0; r < L; ++r) dst[r * L + gl] = f[r];
                 }
-                if (l < le - 1) {
-                    conv2(f);
-                    T s0, s1;
-                    sums(f, s0, s1);
-                    int e0, e1;
-                    const T sc0 = pow2_of(s0, e0), sc1 = pow2_of(s1, e1);
-                    mul_w(f, l + 1, sc0, sc1);
-                }
+            };
+            ck_load(s, f);
+            put(lb);
+            for (int l = lb; l < le - 1; ++l) {
+                conv2(f);
+                T s0, s1;
+                sums(f, s0, s1);
+                int e0, e1;
+                const V sc = {pow2_of(s0, e0), pow2_of(s1, e1)};
+#pragma unroll
+                for (int r = 0; r < L; ++r) f[r] = vmul(f[r], sc);
+                put(l + 1);
+                if (l + 1 < le - 1) mul_w(f, l + 1, T(1), T(1));
             }
             for (int l = le - 1; l >= lb; --l) {
-                // H = G * b and D = dG/dt * b (both end in the layout of F_l)
-                V d[L];
-                {
-                    cvec<V> z[KS], zd[KS];
-                    line_fwd<L>(b, z);
-                    spec_mix<L, false>(zd, z, mixdg);
-                    spec_mix_inplace<L>(z, mixg);
-                    line_inv<L>(z, b);
-                    line_inv<L>(zd, d);
-                }
-                transpose(b);
-                transpose(d);
-                {
-                    cvec<V> z[KS], zd[KS];
-                    line_fwd<L>(b, z);
-                    line_fwd<L>(d, zd);
-                    spec_mix_inplace<L>(zd, mixg);
-                    spec_mix<L, true>(zd, z, mixdg);
-                    spec_mix_inplace<L>(z, mixg);
-                    line_inv<L>(z, b);   // H
-                    line_inv<L>(zd, d);  // D
-                }
-                // F_l from the segment buffer
+                conv2(b);  // H_l = G * b_{l+1}, in the layout of F_l
                 if (active) {
                     const V *src = seg + (long long)(l - lb) * N;
 #pragma unroll
                     for (int r = 0; r < L; ++r) f[r] = src[r * L + gl];
                 }
-                V zf = vzero(b[0]), zdf = vzero(b[0]);
+                // with h = b = H_l: alpha_l where the segment holds it (F_lb at its start, alpha_lb =
+                // F_lb / W_lb), F_l = W_l . alpha_l, b_l = W_l . h
+                T w[L];
+                line_w(l, w);
+                V zd = vzero(b[0]), zf = vzero(b[0]);
+                auto add_across = [&]() {
+                    if (active) {
+#pragma unroll
+                        for (int r = 0; r < L; ++r)
+                            zd = vfma(vmul(b[r], vsplat(w[r])), vadd(f[(r + L - 1) % L], f[(r + 1) % L]), zd);
+                    }
+                };
+                if (l != lb) {
+                    add_across();
+#pragma unroll
+                    for (int r = 0; r < L; ++r) f[r] = vmul(f[r], vsplat(w[r]));
+                }
                 if (active) {
 #pragma unroll
                     for (int r = 0; r < L; ++r) {
                         zf = vfma(f[r], b[r], zf);
-                        zdf = vfma(f[r], d[r], zdf);
+                        zd = vfma(f[r], vadd(b[(r + L - 1) % L], b[(r + 1) % L]), zd);
                     }
                 }
                 const T z0 = group_sum<GW>(zf.x, gmask), z1 = group_sum<GW>(zf.y, gmask);
-                const T zd0 = group_sum<GW>(zdf.x, gmask), zd1 = group_sum<GW>(zdf.y, gmask);
                 if (!(z0 > T(0)) || (has1 && !(z1 > T(0)))) {
                     if (gl == 0) atomicOr(st.status, kStatusNonPositive);
                 }
-                kahan(dts0, dtc0, zd0 / z0);
-                kahan(dts1, dtc1, zd1 / z1);
                 if (dvp && active) {
                     const T iz0 = T(1) / z0, iz1 = has1 ? T(1) / z1 : T(0);
                     T *dvl = dvp + (long long)l * N;
@@ -376,8 +405,17 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                         }
                     }
                 }
-                // b_l = W_l . H_l, renormalised
-                mul_w(b, l, T(1), T(1));
+                if (l == lb && l > 0) {
+#pragma unroll
+                    for (int r = 0; r < L; ++r) f[r] = vmul(f[r], vsplat(T(1) / w[r]));
+                    add_across();
+                }
+                const T zd0 = group_sum<GW>(zd.x, gmask), zd1 = group_sum<GW>(zd.y, gmask);
+                kahan(dts0, dtc0, zd0 / z0);
+                kahan(dts1, dtc1, zd1 / z1);
+#pragma unroll
+                for (int r = 0; r < L; ++r) b[r] = vmul(b[r], vsplat(w[r]));
+                // b_l, renormalised
                 T s0, s1;
                 sums(b, s0, s1);
                 int e0, e1;
@@ -387,7 +425,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                 for (int r = 0; r < L; ++r) b[r] = vmul(b[r], sc);
             }
         }
-        if (gl == 0) atomicAdd(&gk.dt[c], double(dts0) + (has1 ? double(dts1) : 0.0));
+        if (gl == 0) atomicAdd(&gk.dt[c], cd.beta / M * (double(dts0) + (has1 ? double(dts1) : 0.0)));
         __syncwarp(gmask);
     }
     (void)CH;

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) grad_w
         const uint32_t *srow = st.sbits + cd.s_off;
         const uint32_t *scol = srow + (long long)M * L * cd.wpl;
         const T *vlog = vlog_all ? vlog_all + cd.v_off + (long long)sg * M * N : nullptr;
+        const T *wtab = gk.w ? static_cast<const T *>(gk.w) + cd.w_off + (long long)sg * M * N : nullptr;
         T *dvp = dv_all ? dv_all + cd.v_off + (long long)sg * M * N : nullptr;
         const int x0 = st.x[cd.x_off + ((long long)sg * Nsig + pw) * M];
         const int ax = x0 % L, ay = x0 / L;
@@ -104,7 +105,16 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) grad_w
         T v[L];
         // v <- v . W_l . sc  (slice l's layout)
         auto mul_w = [&](int l, T sc) {
-            if (vlog) {
+            if (wtab) {
+                const chunk16_t<T> *src = reinterpret_cast<const chunk16_t<T> *>(wtab + (long long)l * N) + p;
+                static_for<0, L / CH>([&](auto JI) {
+                    constexpr int j = decltype(JI)::value;
+                    T q[CH];
+                    unpack16<0>(q, src[j * L]);
+#pragma unroll
+                    for (int e = 0; e < CH; ++e) v[CH * j + e] *= q[e] * sc;
+                });
+            } else if (vlog) {
                 const T *vl = vlog + (long long)l * N;
 #pragma unroll
                 for (int r = 0; r < L; ++r) v[r] *= exp_t<T>(vl[site(l, r)]) * sc;

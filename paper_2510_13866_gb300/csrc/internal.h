@@ -26,8 +26,6 @@ struct ChainTab {
     // interleaved for k = 0..L/2-1; odd L: ghat(k) for k = 0..L-1
     double mix_d[kMaxL];
     float mix_f[kMaxL];
-    double mixd_d[kMaxL];  // the same for the kernel d g / dt (adjoint)
-    float mixd_f[kMaxL];
     double pplus[2 * kPTab + 1];  // 1 / (1 + e^{-2 lambda m}), m = -kPTab..kPTab
 };
 
@@ -53,6 +51,7 @@ struct ChainDev {
     long long h_off;    // int32 offset of the occupancy histogram [2][M][N]
     long long logw_off; // double offset of log-weights [2][Nsig]
     long long v_off;    // element offset of [2][M][N] gradient arrays
+    long long w_off;    // element offset of the adjoint's exp(v) table (as v_off, 16-byte aligned)
     long long meas_off; // offset into the measurement arrays (N per chain)
     long long perm_off; // int offset of the permutation P [2][Nsig] then its inverse [2][Nsig]
     // windowed backward draw (FP32, Hirsch fields): steps beyond which G is negligible (0: no
@@ -155,6 +154,8 @@ struct GradLaunch {
     void *seg;                 // per group: [K][N] recomputed F_l (context precision pairs)
     long long seg_elems;       // pair elements per group
     const void *v;             // optional log-potential, [2][M][N] per chain (nullable)
+    const void *w;             // exp(v) in the order in which the kernels read it, [2][M][N] at w_off
+                               // (nullable: without the memory for it, exp is taken at every use)
     void *dv;                  // d log Z / d v, same layout (nullable), zeroed by the caller
     double *logz;              // [chain], zeroed by the caller
     double *dt;                // [chain], zeroed by the caller
@@ -185,6 +186,10 @@ cudaError_t launch_local(const DevState &st, int nchains, int max_units, int col
 cudaError_t launch_perm(const DevState &st, int nchains, int max_pairs, cudaStream_t stream);
 
 __device__ __forceinline__ int chain_sign(const DevState &st, int c) { return (st.parity[c] & 1u) ? -1 : 1; }
+// w = exp(v) of the adjoint's log-potential, in the kernels' reading order (max_elems: the largest
+// chain's 2 M N)
+cudaError_t launch_exp_table(const DevState &st, int nchains, long long max_elems, bool fp64, const void *v, void *w,
+                             cudaStream_t stream);
 cudaError_t launch_gauss_w(const DevState &st, int chain, int M, int N, cudaStream_t stream);
 // observables read-out: S(k) and C(r) of every chain; tmp holds 2 N doubles per chain
 cudaError_t launch_readout(const DevState &st, int nchains, int max_N, double *cr_out,

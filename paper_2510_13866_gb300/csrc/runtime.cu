@@ -153,7 +153,9 @@ struct hqmc_ctx {
     int ckpt_kind = HQMC_CKPT_BF16;
     unsigned char *grad_mem = nullptr;
     size_t grad_bytes = 0;
-    long long total_v = 0;
+    void *grad_w = nullptr;  // exp(v) of the last log-potential, where it fits
+    size_t grad_w_bytes = 0;
+    long long total_v = 0, total_w = 0;
 
     // per-phase timing: events [4 * slot]: ffbs start, ffbs end, slice start, slice end
     int prof_max = 0, prof_n = 0;
@@ -214,9 +216,7 @@ void build_tab(const HostChain &h, ChainTab &tb, double lam) {
     }
     // spectral mix of conv_line: with n = L/2, P = (gh_k + gh_{k+n})/2, Q = (gh_k - gh_{k+n})/2,
     // alpha_k = (P - Q sin(2 pi k/L)) / n and beta_k = Q cos(2 pi k/L) / n (gh unnormalised)
-    // (mixd: the same for d gh / dt = 2 dtau cos(2 pi k/L) gh_k)
     auto ghk = [&](double th) { return std::exp(2.0 * z * std::cos(th)); };
-    auto dghk = [&](double th) { return 2.0 * h.dtau * std::cos(th) * std::exp(2.0 * z * std::cos(th)); };
     if (L % 2 == 0) {
         const int n = L / 2;
         for (int k = 0; k < n; ++k) {
@@ -224,19 +224,14 @@ void build_tab(const HostChain &h, ChainTab &tb, double lam) {
             const double P = 0.5 * (ghk(th) + ghk(th2)), Q = 0.5 * (ghk(th) - ghk(th2));
             tb.mix_d[2 * k] = (P - Q * std::sin(th)) / n;
             tb.mix_d[2 * k + 1] = Q * std::cos(th) / n;
-            const double Pd = 0.5 * (dghk(th) + dghk(th2)), Qd = 0.5 * (dghk(th) - dghk(th2));
-            tb.mixd_d[2 * k] = (Pd - Qd * std::sin(th)) / n;
-            tb.mixd_d[2 * k + 1] = Qd * std::cos(th) / n;
         }
     } else {
         for (int k = 0; k < L; ++k) {
             tb.mix_d[k] = ghk(two_pi * k / L) / L;
-            tb.mixd_d[k] = dghk(two_pi * k / L) / L;
         }
     }
     for (int k = 0; k < L; ++k) {
         tb.mix_f[k] = float(tb.mix_d[k]);
-        tb.mixd_f[k] = float(tb.mixd_d[k]);
     }
     std::vector<double> g;
     ring_propagator(L, z, g);
@@ -391,7 +386,7 @@ int plan_layout(hqmc_ctx *c, size_t *total) {
     };
     const size_t o_chains = take(sizeof(ChainDev) * nc);
     const size_t o_tabs = take(sizeof(ChainTab) * nc);
-    long long sb = 0, xb = 0, hb = 0, lb = 0, vb = 0, mb = 0, gb = 0, pb = 0, db = 0, qb = 0;
+    long long sb = 0, xb = 0, hb = 0, lb = 0, vb = 0, wb = 0, mb = 0, gb = 0, pb = 0, db = 0, qb = 0;
     for (int i = 0; i < nc; ++i) {
         const HostChain &h = c->ch[i];
         ChainDev &d = c->cdev[i];
@@ -433,12 +428,15 @@ int plan_layout(hqmc_ctx *c, size_t *total) {
         lb += 2LL * h.Nsig;
         d.v_off = vb;
         vb += 2LL * h.M * h.N;
+        d.w_off = wb;
+        wb += (2LL * h.M * h.N + 3) / 4 * 4;
         d.meas_off = mb;
         mb += h.N;
     }
     c->total_N = size_t(mb);
     c->total_wl = lb;
     c->total_v = vb;
+    c->total_w = wb;
     const size_t o_s = take(size_t(sb) * 4);
     const size_t o_x = take(size_t(xb) * 2);
     const size_t o_h = take(size_t(hb) * 4);
@@ -1581,6 +1579,26 @@ int hqmc_log_weight_grad(hqmc_ctx *c, const void *v, double *logZ, void *dlogZ_d
         c->grad_bytes = off;
     }
     cudaStream_t st = c->stream;
+    if (v) {
+        // exp(v) once for all worldlines; without the memory for it the kernels take it at each use
+        const size_t wsz = size_t(c->total_w) * tsz;
+        if (c->grad_w_bytes < wsz) {
+            if (c->grad_w) cudaFree(c->grad_w);
+            c->grad_w_bytes = 0;
+            if (cudaMalloc(&c->grad_w, wsz) == cudaSuccess) {
+                c->grad_w_bytes = wsz;
+            } else {
+                cudaGetLastError();
+                c->grad_w = nullptr;
+            }
+        }
+        if (c->grad_w) {
+            long long most = 0;
+            for (auto &d : c->cdev) most = std::max(most, 2LL * d.M * d.N);
+            cudaError_t e = launch_exp_table(c->st, c->nchains, most, f64, v, c->grad_w, st);
+            if (e != cudaSuccess) return cuda_fail(c, e, "exp table launch");
+        }
+    }
     double *d_logz = reinterpret_cast<double *>(c->grad_mem);
     double *d_dt = d_logz + c->nchains;
     unsigned *d_next = reinterpret_cast<unsigned *>(d_dt + c->nchains);
@@ -1602,6 +1620,7 @@ int hqmc_log_weight_grad(hqmc_ctx *c, const void *v, double *logZ, void *dlogZ_d
         gk.seg = c->grad_mem + p.off + size_t(p.groups) * p.ck_bytes;
         gk.seg_elems = (long long)p.seg_elems;
         gk.v = v;
+        gk.w = v ? c->grad_w : nullptr;
         gk.dv = dlogZ_dv;
         gk.logz = d_logz;
         gk.dt = d_dt;
@@ -1659,6 +1678,7 @@ void hqmc_destroy(hqmc_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     free_layout(c);
     if (c->grad_mem) cudaFree(c->grad_mem);
+    if (c->grad_w) cudaFree(c->grad_w);
     for (auto s : c->aux) cudaStreamDestroy(s);
     for (auto e : c->ev) cudaEventDestroy(e);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
