@@ -654,14 +654,28 @@ cudaError_t launch_advance(const DevState &st, cudaStream_t stream) {
 //   A[ky][rx] = sum_kx S(kx, ky) cos(2 pi kx rx / L),  B[ky][rx] = sum_kx S(kx, ky) sin(...),
 //   C(rx, ry) = (1/N) sum_ky A[ky][rx] cos(2 pi ky ry / L) - B[ky][rx] sin(2 pi ky ry / L).
 // Phases are reduced mod L before the trigonometric call, so every factor is exact to
-// rounding.  Sums are sign-reweighted (divided by the sum of signs, the sample count
+// rounding.  The L factors are taken once per CTA into shared memory: an FP64 sincospi at every
+// term (the FP64 pipe does two multiply-adds per cycle and SM) was nearly all of the read-out (64
+// chains of L = 32: 227 + 199 us, 14 + 24 us with the table).  Sums are sign-reweighted (divided by the sum of signs, the sample count
 // without permutations).
 // src (nullable): per-chain input in place of the accumulated |m(k)|^2 (the open-path sums
 // for n_k, which take the same separable transform with k and r exchanged)
+__device__ __forceinline__ void phase_table(double2 *tab, int L) {
+    for (int j = threadIdx.x; j < L; j += blockDim.x) {
+        double sn, cs;
+        sincospi(2.0 * double(j) / double(L), &sn, &cs);
+        tab[j] = make_double2(cs, sn);
+    }
+    __syncthreads();
+}
+
 __global__ void readout_rows_kernel(DevState st, const double *src, double *tmp) {
+    __shared__ double2 tab[kMaxL];
     const int c = blockIdx.y;
     const ChainDev &cd = st.chains[c];
     const int L = cd.L, N = cd.N;
+    if (blockIdx.x * blockDim.x >= N) return;
+    phase_table(tab, L);
     const double *sk = (src ? src : st.sk) + cd.meas_off;
     double *A = tmp + 2 * cd.meas_off, *B = A + N;
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < N; o += gridDim.x * blockDim.x) {
@@ -669,10 +683,9 @@ __global__ void readout_rows_kernel(DevState st, const double *src, double *tmp)
         double a = 0.0, b = 0.0;
         int ph = 0;
         for (int kx = 0; kx < L; ++kx) {
-            double sn, cs;
-            sincospi(2.0 * double(ph) / double(L), &sn, &cs);
-            a += sk[ky * L + kx] * cs;
-            b += sk[ky * L + kx] * sn;
+            const double2 w = tab[ph];
+            a += sk[ky * L + kx] * w.x;
+            b += sk[ky * L + kx] * w.y;
             ph += rx;
             if (ph >= L) ph -= L;
         }
@@ -682,9 +695,12 @@ __global__ void readout_rows_kernel(DevState st, const double *src, double *tmp)
 }
 
 __global__ void readout_cols_kernel(DevState st, const double *tmp, double *cr_out, double *sk_out) {
+    __shared__ double2 tab[kMaxL];
     const int c = blockIdx.y;
     const ChainDev &cd = st.chains[c];
     const int L = cd.L, N = cd.N;
+    if (blockIdx.x * blockDim.x >= N) return;
+    phase_table(tab, L);
     const long long ns = st.meas[c].sign_sum;
     const double norm = ns ? 1.0 / (4.0 * double(ns) * cd.M) : 0.0;
     const double *sk = st.sk + cd.meas_off;
@@ -694,9 +710,8 @@ __global__ void readout_cols_kernel(DevState st, const double *tmp, double *cr_o
         double acc = 0.0;
         int ph = 0;
         for (int ky = 0; ky < L; ++ky) {
-            double sn, cs;
-            sincospi(2.0 * double(ph) / double(L), &sn, &cs);
-            acc += A[ky * L + rx] * cs - B[ky * L + rx] * sn;
+            const double2 w = tab[ph];
+            acc += A[ky * L + rx] * w.x - B[ky * L + rx] * w.y;
             ph += ry;
             if (ph >= L) ph -= L;
         }
@@ -718,9 +733,12 @@ cudaError_t launch_readout(const DevState &st, int nchains, int max_N, double *c
 // divided by the sum of signs (Sec. 4, "Observables"; the paper's n_k with
 // sum_x <c^dag_{x+r} c_x> = A(r)): the same two separable passes as C(r)
 __global__ void readout_open_cols_kernel(DevState st, const double *tmp, double *nk_out, double *dm_out) {
+    __shared__ double2 tab[kMaxL];
     const int c = blockIdx.y;
     const ChainDev &cd = st.chains[c];
     const int L = cd.L, N = cd.N;
+    if (blockIdx.x * blockDim.x >= N) return;
+    phase_table(tab, L);
     const long long ns = st.meas[c].sign_sum;
     const double norm = ns ? 1.0 / (double(ns) * N) : 0.0;
     const double *A = tmp + 2 * cd.meas_off, *B = A + N;
@@ -730,9 +748,8 @@ __global__ void readout_open_cols_kernel(DevState st, const double *tmp, double 
         double s = 0.0;
         int ph = 0;
         for (int ry = 0; ry < L; ++ry) {
-            double sn, cs;
-            sincospi(2.0 * double(ph) / double(L), &sn, &cs);
-            s += A[ry * L + kx] * cs - B[ry * L + kx] * sn;
+            const double2 w = tab[ph];
+            s += A[ry * L + kx] * w.x - B[ry * L + kx] * w.y;
             ph += ky;
             if (ph >= L) ph -= L;
         }
