@@ -178,10 +178,11 @@ int slice_group(int max_L, int requested, long long work_slices, int num_sms);
 void window_rule(const ChainTab &tb, int L, double wmax, ChainDev &d);
 void host_chain_table(int L, double t, double U, double dtau, ChainTab &tb, double *lam);
 cudaError_t launch_advance(const DevState &st, cudaStream_t stream);
-// local link updates: the largest (worldline, slice) count of one colour of a chain, and
-// one launch over every chain for one colour (0, 1, 2)
-int local_max_units(int M, int Nsig);
-cudaError_t launch_local(const DevState &st, int nchains, int max_units, int color, cudaStream_t stream);
+// local link updates of every chain (closed: no permutation is in use)
+struct LocalShape {
+    int M, N, Nsig;
+};
+cudaError_t launch_local(const DevState &st, const LocalShape *chains, int nchains, bool closed, cudaStream_t stream);
 // one permutation update (pair swaps at tau = beta) of every chain and spin
 cudaError_t launch_perm(const DevState &st, int nchains, int max_pairs, cudaStream_t stream);
 

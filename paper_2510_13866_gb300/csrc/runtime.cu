@@ -1290,18 +1290,17 @@ int hqmc_local_sweep(hqmc_ctx *c, int n_sweeps) {
     int rc = prepare(c);
     if (rc) return rc;
     HQMC_CUDA(c, cudaSetDevice(c->device));
-    int max_units = 0, max_M = 0, max_L = 0;
+    int max_M = 0, max_L = 0;
+    std::vector<LocalShape> shapes;
     for (auto &d : c->cdev) {
-        max_units = std::max(max_units, local_max_units(d.M, d.Nsig));
+        shapes.push_back({d.M, d.N, d.Nsig});
         max_M = std::max(max_M, d.M);
         max_L = std::max(max_L, d.L);
     }
     for (int i = 0; i < n_sweeps; ++i) {
-        for (int color = 0; color < 3; ++color) {
-            cudaError_t e = launch_local(c->st, c->nchains, max_units, color, c->stream);
-            if (e != cudaSuccess) return cuda_fail(c, e, "local launch");
-        }
-        cudaError_t e = launch_slice(c->st, c->nchains, max_M, max_L, slice_group(max_L, c->slices_per_cta, slice_work(c), c->num_sms), true,
+        cudaError_t e = launch_local(c->st, shapes.data(), c->nchains, !c->perm_used, c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "local launch");
+        e = launch_slice(c->st, c->nchains, max_M, max_L, slice_group(max_L, c->slices_per_cta, slice_work(c), c->num_sms), true,
                                      c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "slice launch");
         e = launch_advance(c->st, c->stream);
