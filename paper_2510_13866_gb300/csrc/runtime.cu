@@ -346,11 +346,23 @@ long long slice_work(const hqmc_ctx *c) {
     return (long long)c->nchains * max_M;
 }
 
+// Warps per CTA of a size class: the caller's or the autotuner's choice, else 4.  An FP64 launch of
+// fewer than four CTAs per SM takes narrower ones, which spread over more SMs: 512 units of L = 16
+// kept 64 of 152 SMs busy with 4 warps each (a sweep of 4 chains, M = 80, 3.27 ms; 2.95 ms with 256
+// CTAs of one warp).  FP32 launches that small are bound by latency, not by a shared pipe, and
+// batches of mixed sizes lost 3% to narrow CTAs, so they keep 4.  Results do not depend on it.
 int default_wpc(hqmc_ctx *c, int L) {
     for (auto &kv : c->class_wpc)
         if (kv.first == L && kv.second > 0) return kv.second;
     if (c->wpc > 0) return c->wpc;
-    return c->precision == HQMC_FP64 ? 4 : 4;
+    if (c->precision != HQMC_FP64) return 4;
+    long long units = 0;
+    for (auto &h : c->ch)
+        if (h.L == L && h.set) units += 2LL * ((h.Nsig + 1) / 2) * ffbs_nblk(h.block, h.M);
+    int w = 4;
+    while (w > 1 && units > 0 && (units + w * ffbs_groups_per_warp(L) - 1) / (w * ffbs_groups_per_warp(L)) < 4LL * c->num_sms)
+        w >>= 1;
+    return w;
 }
 
 // Compute the device layout (offsets) and its size; fills c->classes, c->cdev.
