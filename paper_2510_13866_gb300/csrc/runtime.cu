@@ -64,6 +64,9 @@ struct HostChain {
 // Scratch of a wide FP32 class up to which its CTAs take several slots each: 5% of the device
 constexpr size_t kBatchBytes = size_t(14) << 30;
 
+// Read-backs up to this size go through a context's pinned staging buffer.
+constexpr size_t kPinBytes = size_t(256) << 10;
+
 struct LClass {
     int L = 0;
     std::vector<int> chains;
@@ -133,6 +136,8 @@ struct hqmc_ctx {
 
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+
+    unsigned char *pin = nullptr;  // pinned staging of small read-backs (kPinBytes)
 
     // per-size CTA shape (warps per CTA) chosen by hqmc_set_class_launch / hqmc_autotune
     std::vector<std::pair<int, int>> class_wpc;
@@ -612,6 +617,11 @@ int prepare(hqmc_ctx *c) {
         c->own_mem = true;
     }
     c->bytes = need;
+    if (!c->pin) {
+        void *p = nullptr;
+        if (cudaMallocHost(&p, kPinBytes) == cudaSuccess) c->pin = static_cast<unsigned char *>(p);
+        else cudaGetLastError();  // read-backs then go to pageable memory
+    }
     DevState &s = c->st;
     s.chains = rebase(s.chains, c->base);
     s.tabs = rebase(s.tabs, c->base);
@@ -835,10 +845,48 @@ int enqueue_sweep(hqmc_ctx *c, cudaStream_t st, bool capture) {
     return HQMC_OK;
 }
 
-int check_status(hqmc_ctx *c) {
+// Device arrays read back together, with one synchronisation.  Up to kPinBytes in all they go
+// through the pinned buffer: a copy to pageable memory returns when it is done, so a sweep's
+// log-weights and status, or a chain's field, worldlines, anchor and counter, waited for each other
+// one by one (about 8 us each).
+struct ReadBack {
+    struct Item {
+        void *dst;
+        const void *src;
+        size_t bytes;
+    };
+    std::vector<Item> items;
+    size_t total = 0;
+    void add(void *dst, const void *src, size_t bytes) {
+        items.push_back({dst, src, bytes});
+        total += round_up(bytes, 16);
+    }
+    int run(hqmc_ctx *c) {
+        const bool staged = c->pin && total <= kPinBytes;
+        size_t o = 0;
+        for (auto &it : items) {
+            void *to = staged ? static_cast<void *>(c->pin + o) : it.dst;
+            HQMC_CUDA(c, cudaMemcpyAsync(to, it.src, it.bytes, cudaMemcpyDeviceToHost, c->stream));
+            o += round_up(it.bytes, 16);
+        }
+        HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
+        if (staged) {
+            o = 0;
+            for (auto &it : items) {
+                std::memcpy(it.dst, c->pin + o, it.bytes);
+                o += round_up(it.bytes, 16);
+            }
+        }
+        return HQMC_OK;
+    }
+};
+
+// Runs the read-backs with the status word among them, and reports what the kernels flagged.
+int read_status(hqmc_ctx *c, ReadBack rb = {}) {
     unsigned stt = 0;
-    HQMC_CUDA(c, cudaMemcpyAsync(&stt, c->st.status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    rb.add(&stt, c->st.status, sizeof(unsigned));
+    const int rc = rb.run(c);
+    if (rc) return rc;
     if (stt) {
         HQMC_CUDA(c, cudaMemsetAsync(c->st.status, 0, sizeof(unsigned), c->stream));
         return fail(c, HQMC_ERR_NUMERIC,
@@ -1283,9 +1331,9 @@ int hqmc_sweep(hqmc_ctx *c, int n_sweeps, double *logw_out) {
     }
     c->sweeps_host += n_sweeps;
     if (n_sweeps > 0) c->started = true;
-    if (logw_out)
-        HQMC_CUDA(c, cudaMemcpyAsync(logw_out, c->st.logw, sizeof(double) * c->total_wl, cudaMemcpyDeviceToHost, c->stream));
-    return check_status(c);
+    ReadBack rb;
+    if (logw_out) rb.add(logw_out, c->st.logw, sizeof(double) * c->total_wl);
+    return read_status(c, rb);
 }
 
 int hqmc_logw_error(hqmc_ctx *c, double *err_out) {
@@ -1320,7 +1368,7 @@ int hqmc_local_sweep(hqmc_ctx *c, int n_sweeps) {
     }
     c->sweeps_host += n_sweeps;
     if (n_sweeps > 0) c->started = true;
-    return check_status(c);
+    return read_status(c);
 }
 
 int hqmc_measure(hqmc_ctx *c, hqmc_obs *out, double *Sk, double *Cr, int reset) {
@@ -1331,12 +1379,14 @@ int hqmc_measure(hqmc_ctx *c, hqmc_obs *out, double *Sk, double *Cr, int reset) 
     cudaError_t e = launch_readout(c->st, c->nchains, max_N, c->d_cr, c->d_sko, c->d_rd, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "readout");
     std::vector<MeasAcc> acc(c->nchains);
-    HQMC_CUDA(c, cudaMemcpyAsync(acc.data(), c->st.meas, sizeof(MeasAcc) * c->nchains, cudaMemcpyDeviceToHost, c->stream));
-    if (Sk) HQMC_CUDA(c, cudaMemcpyAsync(Sk, c->d_sko, 8 * c->total_N, cudaMemcpyDeviceToHost, c->stream));
-    if (Cr) HQMC_CUDA(c, cudaMemcpyAsync(Cr, c->d_cr, 8 * c->total_N, cudaMemcpyDeviceToHost, c->stream));
-    std::vector<double> skh(c->total_N);
-    HQMC_CUDA(c, cudaMemcpyAsync(skh.data(), c->d_sko, 8 * c->total_N, cudaMemcpyDeviceToHost, c->stream));
-    HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    std::vector<double> skh(Sk ? 0 : c->total_N);
+    double *sk = Sk ? Sk : skh.data();
+    ReadBack rb;
+    rb.add(acc.data(), c->st.meas, sizeof(MeasAcc) * c->nchains);
+    rb.add(sk, c->d_sko, 8 * c->total_N);
+    if (Cr) rb.add(Cr, c->d_cr, 8 * c->total_N);
+    const int rc = rb.run(c);
+    if (rc) return rc;
     if (out) {
         for (int i = 0; i < c->nchains; ++i) {
             const ChainDev &d = c->cdev[i];
@@ -1353,7 +1403,7 @@ int hqmc_measure(hqmc_ctx *c, hqmc_obs *out, double *Sk, double *Cr, int reset) 
             o.mean_sign = acc[i].samples ? ns / double(acc[i].samples) : 1.0;
             o.n_perm_accepted = (int64_t)acc[i].perm_accepted;
             const int kh = d.L / 2;
-            o.s_pipi = skh[d.meas_off + kh + d.L * kh];
+            o.s_pipi = sk[d.meas_off + kh + d.L * kh];
             o.n_degenerate = (int64_t)acc[i].degenerate;
             o.n_nonpositive = (int64_t)acc[i].nonpositive;
             o.n_local_accepted = (int64_t)acc[i].local_accepted;
@@ -1395,10 +1445,10 @@ int hqmc_measure_open(hqmc_ctx *c, double *nk, double *dm) {
     // the read-out uses the S(k) / C(r) output arrays as its destination
     cudaError_t e = launch_readout_open(c->st, c->nchains, max_N, c->d_cr, c->d_sko, c->d_rd, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "open readout");
-    if (nk) HQMC_CUDA(c, cudaMemcpyAsync(nk, c->d_cr, 8 * c->total_N, cudaMemcpyDeviceToHost, c->stream));
-    if (dm) HQMC_CUDA(c, cudaMemcpyAsync(dm, c->d_sko, 8 * c->total_N, cudaMemcpyDeviceToHost, c->stream));
-    HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
-    return HQMC_OK;
+    ReadBack rb;
+    if (nk) rb.add(nk, c->d_cr, 8 * c->total_N);
+    if (dm) rb.add(dm, c->d_sko, 8 * c->total_N);
+    return rb.run(c);
 }
 
 int hqmc_chain_shape(hqmc_ctx *c, int chain, int *L, int *M, int *Nsig) {
@@ -1415,33 +1465,31 @@ int hqmc_get_state(hqmc_ctx *c, int chain, int8_t *s, int32_t *x, int *anchor, u
     if (rc) return rc;
     const ChainDev &d = c->cdev[chain];
     if (s && d.gauss) std::memset(s, 0, size_t(d.M) * d.N);
+    std::vector<uint32_t> bits;
+    std::vector<int16_t> xs;
+    unsigned long long sw = 0;
+    ReadBack rb;
     if (s && !d.gauss) {
-        std::vector<uint32_t> bits(size_t(d.M) * d.L * d.wpl);
-        HQMC_CUDA(c, cudaMemcpyAsync(bits.data(), c->st.sbits + d.s_off, bits.size() * 4, cudaMemcpyDeviceToHost, c->stream));
-        HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
-        for (int l = 0; l < d.M; ++l)
-            for (int iy = 0; iy < d.L; ++iy)
-                for (int ix = 0; ix < d.L; ++ix) {
-                    const uint32_t w = bits[(size_t(l) * d.L + iy) * d.wpl + (ix >> 5)];
-                    s[size_t(l) * d.N + ix + d.L * iy] = ((w >> (ix & 31)) & 1u) ? 1 : -1;
-                }
+        bits.resize(size_t(d.M) * d.L * d.wpl);
+        rb.add(bits.data(), c->st.sbits + d.s_off, bits.size() * 4);
     }
     if (x) {
-        std::vector<int16_t> xs(2ull * d.Nsig * d.M);
-        HQMC_CUDA(c, cudaMemcpyAsync(xs.data(), c->st.x + d.x_off, xs.size() * 2, cudaMemcpyDeviceToHost, c->stream));
-        HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
-        for (size_t k = 0; k < xs.size(); ++k) x[k] = xs[k];
+        xs.resize(2ull * d.Nsig * d.M);
+        rb.add(xs.data(), c->st.x + d.x_off, xs.size() * 2);
     }
-    if (anchor) {
-        HQMC_CUDA(c, cudaMemcpyAsync(anchor, c->st.anchor + chain, 4, cudaMemcpyDeviceToHost, c->stream));
-        HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (anchor) rb.add(anchor, c->st.anchor + chain, 4);
+    if (sweeps) rb.add(&sw, c->st.sweep, 8);
+    rc = rb.run(c);
+    if (rc) return rc;
+    for (size_t k = 0; k < bits.size(); ++k) {
+        // word k: line iy = (k / wpl) % L of slice k / (wpl L), sites ix = 32 (k % wpl) ..
+        const size_t line = k / d.wpl;
+        const int ix0 = int(k % d.wpl) * 32, n = std::min(32, d.L - ix0);
+        int8_t *out = s + line * d.L + ix0;
+        for (int j = 0; j < n; ++j) out[j] = ((bits[k] >> j) & 1u) ? 1 : -1;
     }
-    if (sweeps) {
-        unsigned long long sw = 0;
-        HQMC_CUDA(c, cudaMemcpyAsync(&sw, c->st.sweep, 8, cudaMemcpyDeviceToHost, c->stream));
-        HQMC_CUDA(c, cudaStreamSynchronize(c->stream));
-        *sweeps = sw;
-    }
+    for (size_t k = 0; k < xs.size(); ++k) x[k] = xs[k];
+    if (sweeps) *sweeps = sw;
     return HQMC_OK;
 }
 
@@ -1642,11 +1690,13 @@ int hqmc_log_weight_grad(hqmc_ctx *c, const void *v, double *logZ, void *dlogZ_d
         if (e != cudaSuccess) return cuda_fail(c, e, "grad launch");
     }
     std::vector<double> h(2 * size_t(c->nchains));
-    HQMC_CUDA(c, cudaMemcpyAsync(h.data(), d_logz, h.size() * 8, cudaMemcpyDeviceToHost, st));
-    HQMC_CUDA(c, cudaStreamSynchronize(st));
+    ReadBack rb;
+    rb.add(h.data(), d_logz, h.size() * 8);
+    rc = read_status(c, rb);
+    if (rc && rc != HQMC_ERR_NUMERIC) return rc;
     if (logZ) std::memcpy(logZ, h.data(), size_t(c->nchains) * 8);
     if (dlogZ_dt) std::memcpy(dlogZ_dt, h.data() + c->nchains, size_t(c->nchains) * 8);
-    return check_status(c);
+    return rc;
 }
 
 int hqmc_set_profiling(hqmc_ctx *c, int max_sweeps) {
@@ -1690,6 +1740,7 @@ void hqmc_destroy(hqmc_ctx *c) {
     free_layout(c);
     if (c->grad_mem) cudaFree(c->grad_mem);
     if (c->grad_w) cudaFree(c->grad_w);
+    if (c->pin) cudaFreeHost(c->pin);
     for (auto s : c->aux) cudaStreamDestroy(s);
     for (auto e : c->ev) cudaEventDestroy(e);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);

@@ -436,7 +436,7 @@ class Lattice:
         self.prepare()
         dt = torch.float64 if self.precision == HQMC_FP64 else torch.float32
         tot = sum(2 * M * L * L for L, M, _ in self.shapes)
-        dv = torch.zeros(tot, dtype=dt, device=f"cuda:{self.device}") if want_dv else None
+        dv = torch.empty(tot, dtype=dt, device=f"cuda:{self.device}") if want_dv else None  # zeroed by the call
         vp = None
         if v is not None:
             if v.dtype != dt or not v.is_cuda or v.numel() != tot:
@@ -480,8 +480,11 @@ def _log_weight_function():
         @staticmethod
         def backward(ctx, g):
             (dv,) = ctx.saved_tensors
-            rep = torch.repeat_interleave(g.to(dv.dtype), torch.as_tensor(ctx.sizes, device=g.device))
-            gv = dv * rep
+            gd = g.to(dv.dtype)
+            if len(set(ctx.sizes)) == 1:
+                gv = (dv.view(len(ctx.sizes), -1) * gd[:, None]).view(-1)
+            else:
+                gv = dv * torch.repeat_interleave(gd, torch.as_tensor(ctx.sizes, device=g.device), output_size=dv.numel())
             gt = None
             if ctx.t_shape is not None:
                 gt = (g.detach().cpu() * ctx.dt).sum().to(torch.float64).reshape(ctx.t_shape)
