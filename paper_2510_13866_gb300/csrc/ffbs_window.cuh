@@ -209,7 +209,7 @@ __device__ __noinline__ int draw_whole(const float *f, const float *g2, int i, i
         const int y = k * SEG + rs;
         const float gy = g2[y - cy + L];
         float p = 0.f;
-#pragma unroll 16
+#pragma unroll 32  // loads in flight: this is the latency of memory, L / 32 times per row
         for (int x = 0; x < L; ++x) p = fmaf(at(x, y), g2[x - cx + L] * gy, p);
         float inc = p;
 #pragma unroll
@@ -240,7 +240,7 @@ __device__ __noinline__ int draw_whole(const float *f, const float *g2, int i, i
         const float gy = g2[win - cy + L];
         float p = 0.f;
         int n = 0;
-#pragma unroll 16
+#pragma unroll 32
         for (int x = 0; x < L; ++x) {
             p = fmaf(at(x, win), g2[x - cx + L] * gy, p);
             n += (p <= rem) ? 1 : 0;

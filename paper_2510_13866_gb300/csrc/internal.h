@@ -170,7 +170,7 @@ size_t ffbs_smem_bytes(int L, bool fp64, int warps_per_cta);
 cudaError_t ffbs_occupancy(int L, bool fp64, int warps_per_cta, int *blocks_per_sm);
 bool ffbs_supported(int L);
 
-cudaError_t launch_init_state(const DevState &st, int nchains, cudaStream_t stream);
+cudaError_t launch_init_state(const DevState &st, int nchains, int max_M, cudaStream_t stream);
 cudaError_t launch_slice(const DevState &st, int nchains, int max_M, int max_L, int slices_per_cta,
                          bool measure, cudaStream_t stream);
 cudaError_t configure_slice(int max_L, int S);

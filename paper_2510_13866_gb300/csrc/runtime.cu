@@ -684,7 +684,9 @@ int prepare(hqmc_ctx *c) {
             HQMC_CUDA(c, cudaMemcpyAsync(s.perm, ident.data(), ident.size() * 4, cudaMemcpyHostToDevice, st));
         HQMC_CUDA(c, cudaStreamSynchronize(st));
     }
-    cudaError_t e = launch_init_state(s, c->nchains, st);
+    int max_M = 0;
+    for (auto &d : c->cdev) max_M = std::max(max_M, d.M);
+    cudaError_t e = launch_init_state(s, c->nchains, max_M, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "init_state");
     HQMC_CUDA(c, cudaStreamSynchronize(st));
     c->sweeps_host = 0;
@@ -1264,12 +1266,17 @@ int hqmc_workspace_size(hqmc_ctx *c, size_t *bytes) {
     auto keep_cdev = c->cdev;
     auto keep_cls = c->classes;
     const bool keep_batch = c->batch_units;
-    // a workspace for the wide classes' extra slots is asked for only where the device has the
-    // room for it (or what is attached already holds it)
-    size_t room = 0, total = 0;
-    HQMC_CUDA(c, cudaSetDevice(c->device));
-    HQMC_CUDA(c, cudaMemGetInfo(&room, &total));
-    int rc = plan_within(c, std::max(room, c->attached_bytes), &need);
+    int rc = plan_within(c, SIZE_MAX, &need);
+    bool extra = false;
+    for (auto &k : c->classes) extra = extra || k.batch > 1;
+    if (!rc && extra) {
+        // the wide classes' extra slots are asked for only where the device has the room for them (or
+        // what is attached already holds them)
+        size_t room = 0, total = 0;
+        HQMC_CUDA(c, cudaSetDevice(c->device));
+        HQMC_CUDA(c, cudaMemGetInfo(&room, &total));
+        rc = plan_within(c, std::max(room, c->attached_bytes), &need);
+    }
     if (c->ready) {
         c->st = keep;
         c->cdev = keep_cdev;

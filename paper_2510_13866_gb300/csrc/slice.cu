@@ -36,6 +36,32 @@ struct SliceSmem {
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
 
+// Integer threshold of a Gibbs draw: with u = k 2^-53 (k the word's leading 53 bits),
+// u < p if and only if k < ceil(p 2^53); p 2^53 is exact.  The draws then take no FP64 operation per
+// site (two per cycle and SM).  With div_n and the unrolled transforms below the kernel takes 161
+// instead of 177 us for 64 chains of L = 32 (M = 80), the grouped form 37.5 instead of 43.5 us for
+// 32 of L = 12 (M = 120).
+__device__ __forceinline__ unsigned long long gibbs_threshold(double p) { return (unsigned long long)ceil(p * 0x1.0p53); }
+
+// x / N for an integer N < 2^15 with inv = 1 / N correctly rounded: the correctly rounded quotient by
+// one residual (Markstein, IBM J. Res. Dev. 34, 1990), exact in one product when N is a power of two.
+__device__ __forceinline__ double div_n(double x, double n, double inv, bool pow2) {
+    const double q = x * inv;
+    return pow2 ? q : fma(fma(-q, n, x), inv, q);
+}
+
+// One term of the direct transform of a line: z += a w, for a real a and for a complex one (the
+// order of the roundings is spelled out: it is part of S(k)'s last bits).
+__device__ __forceinline__ void dft_real(float2 &z, float a, float2 w) {
+    z.x = fmaf(a, w.x, z.x);
+    z.y = fmaf(a, w.y, z.y);
+}
+__device__ __forceinline__ void dft_complex(float2 &z, float2 a, float2 w) {
+    z.x = __fadd_rn(z.x, fmaf(a.x, w.x, -__fmul_rn(a.y, w.y)));
+    z.y = __fadd_rn(z.y, fmaf(a.y, w.x, __fmul_rn(a.x, w.y)));
+}
+__device__ __forceinline__ float norm2(float2 z) { return fmaf(z.x, z.x, __fmul_rn(z.y, z.y)); }
+
 // byte offsets of the slice kernel's shared arrays for lattice size L and S slices handled
 // together: per slice the field bits by rows and columns, the slice's m and its row DFT,
 // and (grouped form) its |m^(k)|^2 before the sum over the group's slices
@@ -108,14 +134,16 @@ __global__ void __launch_bounds__(kSliceThreads) slice_kernel(DevState st, int s
     uint32_t *rows = reinterpret_cast<uint32_t *>(smem_raw + lay.rows);  // [L][wpl]
     uint32_t *cols = rows + L * wpl;                                     // [L][wpl]
     unsigned long long *red = reinterpret_cast<unsigned long long *>(smem_raw + lay.red);
-    double *pp = reinterpret_cast<double *>(smem_raw + lay.pp);         // P(s=+1 | m), |m| <= kPTab
+    unsigned long long *pp = reinterpret_cast<unsigned long long *>(smem_raw + lay.pp);  // thresholds, |m| <= kPTab
+    const double dn = double(N), inv_n = 1.0 / dn;
+    const bool pow2 = (N & (N - 1)) == 0;
     float *ms = reinterpret_cast<float *>(smem_raw + lay.ms);            // [N] m of the slice
     float2 *x1 = reinterpret_cast<float2 *>(smem_raw + lay.x1);          // [N] row DFT
     float2 *tw = reinterpret_cast<float2 *>(smem_raw + lay.tw);          // [L] e^{-2 pi i j / L}
     double *skacc = reinterpret_cast<double *>(smem_raw + lay.sk);       // [N]
 
     for (int k = threadIdx.x; k < 2 * L * wpl; k += blockDim.x) rows[k] = 0u;
-    for (int k = threadIdx.x; k < 2 * kPTab + 1; k += blockDim.x) pp[k] = tb.pplus[k];
+    for (int k = threadIdx.x; k < 2 * kPTab + 1; k += blockDim.x) pp[k] = gibbs_threshold(tb.pplus[k]);
     if (do_sk) {
         for (int j = threadIdx.x; j < L; j += blockDim.x) {
             float s, co;
@@ -189,9 +217,9 @@ __global__ void __launch_bounds__(kSliceThreads) slice_kernel(DevState st, int s
                 if (x >= N) break;
                 const int nu = nuq[j], nd = ndq[j];
                 const int m = nu - nd;
-                const double pplus = (m >= -kPTab && m <= kPTab) ? pp[m + kPTab]
-                                                                  : 1.0 / (1.0 + exp(-2.0 * lam * m));
-                const bool up = u53(w4.v[j]) < pplus;
+                const unsigned long long thr = (m >= -kPTab && m <= kPTab) ? pp[m + kPTab]
+                                                                           : gibbs_threshold(1.0 / (1.0 + exp(-2.0 * lam * m)));
+                const bool up = (w4.v[j] >> 11) < thr;
                 const int ix = x % L, iy = x / L;
                 if (up) {
                     atomicOr(&rows[iy * wpl + (ix >> 5)], 1u << (ix & 31));
@@ -217,16 +245,16 @@ __global__ void __launch_bounds__(kSliceThreads) slice_kernel(DevState st, int s
             // x1[iy][kx] = sum_ix m[iy][ix] e^{-2 pi i kx ix / L}
             for (int o = threadIdx.x; o < K1 * L; o += blockDim.x) {
                 const int kx = o % K1, iy = o / K1;
-                float re = 0.f, im = 0.f;
+                const float *row = ms + iy * L;
+                float2 z = make_float2(0.f, 0.f);
                 int ph = 0;
+#pragma unroll 8
                 for (int ix = 0; ix < L; ++ix) {
-                    const float mv = ms[iy * L + ix];
-                    re += mv * tw[ph].x;
-                    im += mv * tw[ph].y;
+                    dft_real(z, row[ix], tw[ph]);
                     ph += kx;
                     if (ph >= L) ph -= L;
                 }
-                x1[o] = make_float2(re, im);
+                x1[o] = z;
             }
         }
         __syncthreads();
@@ -235,16 +263,16 @@ __global__ void __launch_bounds__(kSliceThreads) slice_kernel(DevState st, int s
             // m^[ky][kx] = sum_iy x1[iy][kx] e^{-2 pi i ky iy / L};  S += |m^|^2 / N
             for (int o = threadIdx.x; o < K1 * L; o += blockDim.x) {
                 const int kx = o % K1, ky = o / K1;
-                float re = 0.f, im = 0.f;
+                const float2 *col = x1 + kx;
+                float2 z = make_float2(0.f, 0.f);
                 int ph = 0;
+#pragma unroll 8
                 for (int iy = 0; iy < L; ++iy) {
-                    const float2 a = x1[iy * K1 + kx], w = tw[ph];
-                    re += a.x * w.x - a.y * w.y;
-                    im += a.x * w.y + a.y * w.x;
+                    dft_complex(z, col[iy * K1], tw[ph]);
                     ph += ky;
                     if (ph >= L) ph -= L;
                 }
-                const double v = double(re * re + im * im) / double(N);
+                const double v = div_n(double(norm2(z)), dn, inv_n, pow2);
                 const int k = ky * L + kx;
                 const bool mirror = kx > 0 && 2 * kx < L;
                 const int km = (ky == 0 ? 0 : L - ky) * L + (L - kx);
@@ -303,7 +331,9 @@ __global__ void __launch_bounds__(kSliceThreads) slice_group_kernel(DevState st,
     const SliceSmem lay = slice_smem_layout(L, wpl, S, true);
     uint32_t *rows = reinterpret_cast<uint32_t *>(smem_raw + lay.rows);  // [S][2][L][wpl]
     unsigned long long *red = reinterpret_cast<unsigned long long *>(smem_raw + lay.red);
-    double *pp = reinterpret_cast<double *>(smem_raw + lay.pp);         // P(s=+1 | m), |m| <= kPTab
+    unsigned long long *pp = reinterpret_cast<unsigned long long *>(smem_raw + lay.pp);  // thresholds, |m| <= kPTab
+    const double dn = double(N), inv_n = 1.0 / dn;
+    const bool pow2 = (N & (N - 1)) == 0;
     float *ms = reinterpret_cast<float *>(smem_raw + lay.ms);            // [S][N] m of the slices
     float2 *x1 = reinterpret_cast<float2 *>(smem_raw + lay.x1);          // [S][L][K1] row DFTs
     float2 *tw = reinterpret_cast<float2 *>(smem_raw + lay.tw);          // [L] e^{-2 pi i j / L}
@@ -311,7 +341,7 @@ __global__ void __launch_bounds__(kSliceThreads) slice_group_kernel(DevState st,
     const int bits = 2 * L * wpl;  // words of one slice's rows and columns
 
     for (int k = threadIdx.x; k < ns * bits; k += blockDim.x) rows[k] = 0u;
-    for (int k = threadIdx.x; k < 2 * kPTab + 1; k += blockDim.x) pp[k] = tb.pplus[k];
+    for (int k = threadIdx.x; k < 2 * kPTab + 1; k += blockDim.x) pp[k] = gibbs_threshold(tb.pplus[k]);
     if (do_sk) {
         for (int j = threadIdx.x; j < L; j += blockDim.x) {
             float sn, co;
@@ -389,9 +419,9 @@ __global__ void __launch_bounds__(kSliceThreads) slice_group_kernel(DevState st,
                 if (x >= N) break;
                 const int nu = nuq[j], nd = ndq[j];
                 const int m = nu - nd;
-                const double pplus = (m >= -kPTab && m <= kPTab) ? pp[m + kPTab]
-                                                                  : 1.0 / (1.0 + exp(-2.0 * lam * m));
-                const bool up = u53(w4.v[j]) < pplus;
+                const unsigned long long thr = (m >= -kPTab && m <= kPTab) ? pp[m + kPTab]
+                                                                           : gibbs_threshold(1.0 / (1.0 + exp(-2.0 * lam * m)));
+                const bool up = (w4.v[j] >> 11) < thr;
                 const int ix = x % L, iy = x / L;
                 if (up) {
                     atomicOr(&rw[iy * wpl + (ix >> 5)], 1u << (ix & 31));
@@ -423,16 +453,15 @@ __global__ void __launch_bounds__(kSliceThreads) slice_group_kernel(DevState st,
             const int sl = o / (K1 * L), r = o - sl * (K1 * L);
             const int kx = r % K1, iy = r / K1;
             const float *msl = ms + sl * N + iy * L;
-            float re = 0.f, im = 0.f;
+            float2 z = make_float2(0.f, 0.f);
             int ph = 0;
+#pragma unroll 4
             for (int ix = 0; ix < L; ++ix) {
-                const float mv = msl[ix];
-                re += mv * tw[ph].x;
-                im += mv * tw[ph].y;
+                dft_real(z, msl[ix], tw[ph]);
                 ph += kx;
                 if (ph >= L) ph -= L;
             }
-            x1[o] = make_float2(re, im);
+            x1[o] = z;
         }
         __syncthreads();
         // m^[ky][kx] = sum_iy x1[iy][kx] e^{-2 pi i ky iy / L} for every (slice, k) of the
@@ -443,16 +472,15 @@ __global__ void __launch_bounds__(kSliceThreads) slice_group_kernel(DevState st,
             const int sl = o / (K1 * L), r = o - sl * (K1 * L);
             const int kx = r % K1, ky = r / K1;
             const float2 *xs = x1 + sl * (K1 * L);
-            float re = 0.f, im = 0.f;
+            float2 z = make_float2(0.f, 0.f);
             int ph = 0;
+#pragma unroll 4
             for (int iy = 0; iy < L; ++iy) {
-                const float2 a = xs[iy * K1 + kx], w = tw[ph];
-                re += a.x * w.x - a.y * w.y;
-                im += a.x * w.y + a.y * w.x;
+                dft_complex(z, xs[iy * K1 + kx], tw[ph]);
                 ph += ky;
                 if (ph >= L) ph -= L;
             }
-            vb[o] = double(re * re + im * im) / double(N);
+            vb[o] = div_n(double(norm2(z)), dn, inv_n, pow2);
         }
         __syncthreads();
         for (int o = threadIdx.x; o < K1 * L; o += blockDim.x) {
@@ -584,8 +612,9 @@ __global__ void init_paths_kernel(DevState st) {
     if (sg == 0) st.anchor[c] = -1;
 }
 
-cudaError_t launch_init_state(const DevState &st, int nchains, cudaStream_t stream) {
-    init_fields_kernel<<<dim3(1, nchains), 256, 0, stream>>>(st);
+cudaError_t launch_init_state(const DevState &st, int nchains, int max_M, cudaStream_t stream) {
+    // a CTA per slice (one CTA per chain took 6.9 ms for two chains of L = 128, M = 160)
+    init_fields_kernel<<<dim3(std::min(max_M, 256), nchains), 256, 0, stream>>>(st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     init_paths_kernel<<<nchains, 32, 0, stream>>>(st);
