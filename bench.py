@@ -353,7 +353,7 @@ def kernel_source_digest(workload="L32"):
     import re
 
     h = hashlib.sha256()
-    files = ("ffbs.cuh", "device_common.cuh") if workload == "L32" else ("ffbs.cuh", "ffbs_wide.cuh",
+    files = ("ffbs.cuh", "device_common.cuh") if workload == "L32" else ("ffbs.cuh", "ffbs_wide.cuh", "ffbs_window.cuh",
                                                                           "device_common.cuh")
     for f in files:
         with open(os.path.join(ROOT, "paper_2510_13866_gb300", "csrc", f)) as fh:
@@ -493,9 +493,9 @@ def main():
     ffbs_avg = ffbs_ms / max(1, nprof)
     slice_avg = slice_ms / max(1, nprof)
     # algorithmic work per launch: every particle-slice writes f_l (4N B) and reads it back
-    # (4N B); 5 N log2 N + 4 N flops
+    # (4N B, or on wide lattices a window of 25 x 28 sites); 5 N log2 N + 4 N flops
     part_slices = sum(2 * ns * M for (_, M, ns) in shapes)
-    alg_bytes = sum(2 * ns * M * 8.0 * L * L for (L, M, ns) in shapes)
+    alg_bytes = sum(2 * ns * M * (4.0 * L * L + (2800.0 if L > 32 else 4.0 * L * L)) for (L, M, ns) in shapes)
     alg_flops = sum(2 * ns * M * (5.0 * L * L * np.log2(L * L) + 4.0 * L * L) for (L, M, ns) in shapes)
     ckpt_note = None
     if args.fstore != "stream" and max(Ls) > 32:
@@ -531,6 +531,13 @@ def main():
                 "alg_bytes_per_launch": alg_bytes,
                 "alu": {"achieved_tflops": achieved_flops, "peak_tflops": peak_alu,
                         "frac": achieved_flops / peak_alu, "peak_source": alu_src}}
+    if ckpt_note is None and min(Ls) > 32:
+        # with the backward pass reading windows, the FFTs bound the wide kernel: the ALU figures
+        # lead, the bytes stand beside them
+        roofline.update({"bound": "alu", "achieved": achieved_flops, "peak": peak_alu, "unit": "TFLOP/s",
+                         "frac": achieved_flops / peak_alu, "peak_source": alu_src,
+                         "hbm": {"achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
+                                 "peak_source": peak_src}})
     if ckpt_note is not None:
         # the recompute makes the checkpoint form an FP32-ALU-bound filter: the ALU figures
         # lead, the bytes stand beside them

@@ -23,8 +23,15 @@
 
 namespace hqmc {
 
+// Resident CTAs per SM the adjoint's registers are sized for: as the FFBS kernel's, but four at L = 48
+// in FP32 (168 registers without spills; at six, 96 registers and 888 bytes of spill, 2 chains of
+// M = 40 and 300 worldlines per spin took 1.62 ms instead of 1.41).  At L = 64 the spills of eight
+// CTAs (128 registers) cost less than four CTAs' lost warps (3.37 against 3.73 ms at 512 worldlines).
 template <typename T, int L>
-__global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) grad_wide_kernel(DevState st, GradLaunch gk) {
+constexpr int kGradMinBlocks = (sizeof(T) == 4 && L == 48) ? 4 : WideGeo<T, L>::MINB;
+
+template <typename T, int L>
+__global__ void __launch_bounds__(WideGeo<T, L>::NT, kGradMinBlocks<T, L>) grad_wide_kernel(DevState st, GradLaunch gk) {
     using G = WideGeo<T, L>;
     constexpr int WPC = G::WPC, NT = G::NT, NW = G::NW, CH = G::CH, LP = G::LP, N = L * L;
     extern __shared__ __align__(16) unsigned char smem_raw[];
