@@ -73,3 +73,31 @@ def test_window_edges(L, M, dtau, t):
     """One to four slices (fewer than the windows loaded ahead), no hopping, and hops too long
     for a window (t dtau above 0.14: whole slices in both)."""
     assert_same(sweeps(L, 3, M, dtau, "stream", t=t), sweeps(L, 3, M, dtau, "f32", t=t))
+
+
+def test_workspace_without_extra_slots_gives_the_same_sweep():
+    """hqmc_workspace_size asks for several scratch slots per CTA where units outnumber CTAs; an attached
+    workspace of the size without them is accepted and draws the same, a smaller one is refused."""
+    import ctypes as C
+
+    import torch
+
+    from paper_2510_13866_gb300 import Lattice, hqmc
+
+    def run(fraction):
+        lat = Lattice(64, [5], precision="fp32", torch_memory=False)
+        lat.set_params(1.0, 4.0, 0.25, 0.05, 1400 / 4096)  # 1400 units of one worldline, M = 5
+        n = int(lat.workspace_size() * fraction) // 256 * 256
+        ws = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+        p = (ws.data_ptr() + 255) // 256 * 256
+        rc = hqmc.lib().hqmc_attach_workspace(lat._ctx, C.c_void_p(p), n)
+        out = None if rc else [lat.sweep(2, logw=True)[0].copy(), lat.get_state(0)[1]]
+        lat.close()
+        return rc, out
+
+    rc, full = run(1.0)
+    assert rc == 0
+    rc, small = run(0.65)
+    assert rc == 0
+    assert all(np.array_equal(a, b) for a, b in zip(full, small))
+    assert run(0.2)[0] == -2  # HQMC_ERR_NOMEM
