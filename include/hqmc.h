@@ -157,8 +157,11 @@ int hqmc_set_block(hqmc_ctx *ctx, int chain, int B);
 #define HQMC_FSTORE_F32 2
 int hqmc_set_ffbs_storage(hqmc_ctx *ctx, int kind, int stride);
 
-/* CUDA stream (a cudaStream_t passed as void*) on which every later call is ordered;
- * NULL = the legacy default stream.  Changing it drops the captured sweep graph. */
+/* CUDA stream (a cudaStream_t passed as void*) on which every later call is ordered; NULL (and a
+ * new context) = a non-blocking stream of the context's own.  On that one, the calls that take
+ * device memory (hqmc_attach_workspace, hqmc_log_weight_grad) use it after everything that was
+ * queued on the legacy default stream before the call; work on another stream is the caller's to
+ * wait for.  Changing the stream drops the captured sweep graph. */
 int hqmc_set_stream(hqmc_ctx *ctx, void *stream);
 
 /* Launch configuration: use_graph = replay one captured CUDA graph per sweep;

@@ -106,6 +106,7 @@ struct hqmc_ctx {
     bool own_stream = false;
     std::vector<cudaStream_t> aux;
     std::vector<cudaEvent_t> ev;
+    cudaEvent_t ev_default = nullptr;  // the legacy default stream's work at a hand-over of device memory
     bool use_graph = true, persistent = true;
     int wpc = 0;
     int slices_per_cta = 0;  // Gibbs/measure kernel: slices handled by one CTA (0: automatic)
@@ -589,6 +590,18 @@ int plan_within(hqmc_ctx *c, size_t limit, size_t *need) {
     return plan_layout(c, need);
 }
 
+// What is queued on the legacy default stream so far comes before what the context enqueues from here on.
+// A context whose stream was given as NULL runs on a non-blocking stream of its own, which does not wait for the
+// default stream by itself; the device memory that a caller hands over (a workspace, v, dlogZ_dv) may still be
+// written or read there.
+int after_default_stream(hqmc_ctx *c) {
+    if (!c->own_stream) return HQMC_OK;
+    if (!c->ev_default) HQMC_CUDA(c, cudaEventCreateWithFlags(&c->ev_default, cudaEventDisableTiming));
+    HQMC_CUDA(c, cudaEventRecord(c->ev_default, cudaStreamLegacy));
+    HQMC_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_default, 0));
+    return HQMC_OK;
+}
+
 // Plan, bind memory (attached or owned), upload tables and initialise the state.
 int prepare(hqmc_ctx *c) {
     if (c->ready) return HQMC_OK;
@@ -600,6 +613,8 @@ int prepare(hqmc_ctx *c) {
         if (c->attached_bytes < need) return fail(c, HQMC_ERR_NOMEM, "attached workspace too small");
         c->base = c->attached;
         c->own_mem = false;
+        rc = after_default_stream(c);
+        if (rc) return rc;
     } else {
         void *p = nullptr;
         cudaError_t e = cudaMalloc(&p, need);
@@ -1644,6 +1659,8 @@ int hqmc_log_weight_grad(hqmc_ctx *c, const void *v, double *logZ, void *dlogZ_d
         c->grad_mem = static_cast<unsigned char *>(m);
         c->grad_bytes = off;
     }
+    rc = after_default_stream(c);
+    if (rc) return rc;
     cudaStream_t st = c->stream;
     if (v) {
         // exp(v) once for all worldlines; without the memory for it the kernels take it at each use
@@ -1750,6 +1767,7 @@ void hqmc_destroy(hqmc_ctx *c) {
     if (c->pin) cudaFreeHost(c->pin);
     for (auto s : c->aux) cudaStreamDestroy(s);
     for (auto e : c->ev) cudaEventDestroy(e);
+    if (c->ev_default) cudaEventDestroy(c->ev_default);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }

@@ -144,8 +144,8 @@ class Lattice:
         self._ctx = C.c_void_p()
         self._check(lib().hqmc_init_lattice(C.byref(self._ctx), self.n_chains, _ptr(self.Ls),
                                             _ptr(self.seeds), self.precision, device), ctx=False)
-        stream = torch.cuda.current_stream(device)
-        self._check(lib().hqmc_set_stream(self._ctx, C.c_void_p(stream.cuda_stream)))
+        self._stream = torch.cuda.current_stream(device).cuda_stream
+        self._check(lib().hqmc_set_stream(self._ctx, C.c_void_p(self._stream)))
         self.shapes = None
         self.params = None
         # (t, U, beta, dtau, filling) of every chain as last set, so that a change of t
@@ -266,12 +266,21 @@ class Lattice:
         self._check(lib().hqmc_workspace_size(self._ctx, C.byref(n)))
         return n.value
 
+    def _order(self):
+        """Before device memory goes to the library: torch's work on the current stream comes first.
+        The library waits for the default stream itself where it was given none; a stream other
+        than the context's is waited for here."""
+        cur = self._torch.cuda.current_stream(self.device)
+        if cur.cuda_stream != self._stream:
+            cur.synchronize()
+
     def _attach(self):
         n = self.workspace_size()
         if self._ws is None or self._ws.numel() < n:
             self._ws = self._torch.empty(n + 256, dtype=self._torch.uint8, device=f"cuda:{self.device}")
         p = self._ws.data_ptr()
         p = (p + 255) // 256 * 256
+        self._order()
         self._check(lib().hqmc_attach_workspace(self._ctx, C.c_void_p(p), n))
 
     def prepare(self):
@@ -445,6 +454,7 @@ class Lattice:
             vp = C.c_void_p(v.data_ptr())
         lz = np.zeros(self.n_chains)
         ddt = np.zeros(self.n_chains)
+        self._order()
         self._check(lib().hqmc_log_weight_grad(self._ctx, vp, _ptr(lz),
                                                None if dv is None else C.c_void_p(dv.data_ptr()), _ptr(ddt)))
         return lz, dv, ddt
