@@ -23,6 +23,9 @@
 //     <F_l, (dG/dt) * b_{l+1}> = dtau (<F_l, A_r H_l> + <A_c alpha_{l+1}, b_{l+1}>),
 // where r is the direction that slice l's layout keeps in registers and c the other one, which
 // slice l + 1's layout keeps in registers: both sums are over neighbours in a lane's own line.
+// At the first slice of a segment alpha_l is F_l / W_l; a slice with a site where W_l vanishes (a
+// masked site, v = -inf) or comes near takes its second sum from alpha_l itself instead, which the
+// segment before it then recomputes one step further.
 // Carrying (dG/dt) * b as a second message took 7 half-length FFTs and two transposes per reverse
 // slice instead of 4 and one.  The kernel is bound by the FMA pipe: L = 16, M = 80, 128 chains with a
 // given v, 2.87 ms before this and exp_table_kernel, 2.17 ms with both (and 35 us for the table).
@@ -42,6 +45,11 @@ struct GradGeo {
     static constexpr size_t MIXB = F::MIXB;
     static constexpr size_t GROUP_BYTES = XBUF + MIXB;
 };
+
+// The least W by which a checkpointed F = W alpha is divided to give alpha.  From here on 1 / W is
+// normal, and so is F (in BF16 too) for alpha above 2^-66 of its slice's sum, which is far below the
+// rounding of the transforms.
+constexpr float kDivideMin = 0x1.0p-60f;
 
 template <typename T>
 __device__ __forceinline__ T exp_t(T x);
@@ -319,6 +327,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
             sum = t;
         };
         const int nseg = (M + K - 1) / K;
+        bool late = false;  // the sum over alpha of the slice after this segment is still to be taken
         for (int s = nseg - 1; s >= 0; --s) {
             const int lb = s * K, le = min(M, lb + K);
             // recompute the segment (same lane, same slots): F_lb from its checkpoint, then
@@ -332,7 +341,8 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
             };
             ck_load(s, f);
             put(lb);
-            for (int l = lb; l < le - 1; ++l) {
+            const int lt = late ? le : le - 1;
+            for (int l = lb; l < lt; ++l) {
                 conv2(f);
                 T s0, s1;
                 sums(f, s0, s1);
@@ -340,8 +350,22 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                 const V sc = {pow2_of(s0, e0), pow2_of(s1, e1)};
 #pragma unroll
                 for (int r = 0; r < L; ++r) f[r] = vmul(f[r], sc);
-                put(l + 1);
-                if (l + 1 < le - 1) mul_w(f, l + 1, T(1), T(1));
+                if (l + 1 < le) put(l + 1);
+                if (l + 1 < lt) mul_w(f, l + 1, T(1), T(1));
+            }
+            if (late) {
+                // <A_c alpha_le, b_le> / Z with Z = <alpha_le, b_le>
+                V z = vzero(b[0]), zd = vzero(b[0]);
+                if (active) {
+#pragma unroll
+                    for (int r = 0; r < L; ++r) {
+                        z = vfma(f[r], b[r], z);
+                        zd = vfma(b[r], vadd(f[(r + L - 1) % L], f[(r + 1) % L]), zd);
+                    }
+                }
+                kahan(dts0, dtc0, group_sum<GW>(zd.x, gmask) / group_sum<GW>(z.x, gmask));
+                kahan(dts1, dtc1, group_sum<GW>(zd.y, gmask) / group_sum<GW>(z.y, gmask));
+                late = false;
             }
             for (int l = le - 1; l >= lb; --l) {
                 conv2(b);  // H_l = G * b_{l+1}, in the layout of F_l
@@ -406,9 +430,15 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
                     }
                 }
                 if (l == lb && l > 0) {
+                    bool divide = true;
 #pragma unroll
-                    for (int r = 0; r < L; ++r) f[r] = vmul(f[r], vsplat(T(1) / w[r]));
-                    add_across();
+                    for (int r = 0; r < L; ++r) divide = divide && w[r] >= T(kDivideMin);
+                    late = !__all_sync(gmask, divide);
+                    if (!late) {
+#pragma unroll
+                        for (int r = 0; r < L; ++r) f[r] = vmul(f[r], vsplat(T(1) / w[r]));
+                        add_across();
+                    }
                 }
                 const T zd0 = group_sum<GW>(zd.x, gmask), zd1 = group_sum<GW>(zd.y, gmask);
                 kahan(dts0, dtc0, zd0 / z0);
