@@ -84,9 +84,10 @@ __device__ __forceinline__ float link_h(const float *h, int L, Site a, Site b) {
 
 // One move of slice l of a worldline at x between xm and xn, with the words of its step and its
 // acceptance: returns the final site.  The decision u < R is the FP64 one.  FP32 decides it where u
-// and R lie further apart than its error: the factors of the direction that does not move cancel,
-// and four table values, their products and one division leave R within 2e-6 of itself, the leading
-// 24 bits leave u within 2^-24.  All but about 1e-5 of the moves end there; the FP64 form took its
+// and R lie further apart than its error: the factors of the direction that does not move cancel
+// (where they are so small that the FP64 products could underflow, FP64 decides), and four table
+// values, their products and one division leave R within 2e-6 of itself, the leading 24 bits leave u
+// within 2^-24.  All but about 1e-5 of the moves end there; the FP64 form took its
 // 25 FP64 operations (two per cycle and SM) for every one.
 __device__ __forceinline__ int local_move(const DevState &st, const ChainDev &cd, const ChainTab &tb, const LocalTab &lt, int sg,
                                           int l, int x, int xm, int xn, uint64_t wstep, uint64_t wacc, unsigned magic,
@@ -105,14 +106,17 @@ __device__ __forceinline__ int local_move(const DevState &st, const ChainDev &cd
         const uint32_t *rows = st.sbits + cd.s_off + (long long)l * L * cd.wpl;
         const uint32_t w0 = rows[s.y * cd.wpl + (s.x >> 5)], w1 = rows[n.y * cd.wpl + (n.x >> 5)];
         float num = lt.w[sg][(w1 >> (n.x & 31)) & 1u], den = lt.w[sg][(w0 >> (s.x & 31)) & 1u];
+        float held = 1.f;  // the factors that cancel
         if (M > 1) {
             const bool ydir = dir >= 2;
             const int p = ydir ? s.y : s.x, q = ydir ? n.y : n.x, pa = ydir ? a.y : a.x, pb = ydir ? b.y : b.x;
+            const int o = ydir ? s.x : s.y, oa = ydir ? a.x : a.y, ob = ydir ? b.x : b.y;
+            held = lt.g[wrapd(o - oa, L)] * lt.g[wrapd(ob - o, L)];
             num *= lt.g[wrapd(q - pa, L)] * lt.g[wrapd(pb - q, L)];
             den *= lt.g[wrapd(p - pa, L)] * lt.g[wrapd(pb - p, L)];
         }
         const float R = num / den, u = float(uint32_t(wacc >> 40)) * 0x1.0p-24f;
-        if (num > 1e-30f && den > 1e-30f && R < 1e30f && fabsf(u - R) > 4e-6f * R + 1.2e-7f) {
+        if (num > 1e-30f && den > 1e-30f && R < 1e30f && held > 1e-30f && held < 1e30f && fabsf(u - R) > 4e-6f * R + 1.2e-7f) {
             accepted = u < R;
             sure = true;
         }
@@ -231,7 +235,7 @@ __global__ void __launch_bounds__(kPairThreads) local_pairs_kernel(DevState st, 
                 }
                 const int xf = local_move(st, cd, tb, lt, sg, l, xp[l], xm, xn, ws, wa, magic, accepted);
                 if (accepted) xp[l] = int16_t(xf);
-                        if (color) {
+                if (color) {
                     const Site a = site_of(xm, L, magic), f = site_of(xf, L, magic), b = site_of(xn, L, magic);
                     ek += link_h(lt.h, L, a, f);
                     if (local_color(M, ln) == 0) ek += link_h(lt.h, L, f, b);
