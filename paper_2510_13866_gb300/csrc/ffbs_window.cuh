@@ -25,6 +25,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "window_rule.h"
 
 namespace hqmc {
 

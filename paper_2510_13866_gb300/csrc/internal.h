@@ -10,7 +10,6 @@ namespace hqmc {
 
 constexpr int kMaxL = 128;
 constexpr int kPTab = 64;  // P(s=+1 | m) tabulated for |m| <= kPTab, computed beyond
-constexpr int kWinHalf = 12;  // half width of the backward draw's window (ffbs_window.cuh)
 
 // Per-chain tables, computed on the host in FP64 at set_params.
 struct ChainTab {
@@ -175,7 +174,6 @@ cudaError_t launch_slice(const DevState &st, int nchains, int max_M, int max_L, 
                          bool measure, cudaStream_t stream);
 cudaError_t configure_slice(int max_L, int S);
 int slice_group(int max_L, int requested, long long work_slices, int num_sms);
-void window_rule(const ChainTab &tb, int L, double wmax, ChainDev &d);
 void host_chain_table(int L, double t, double U, double dtau, ChainTab &tb, double *lam);
 cudaError_t launch_advance(const DevState &st, cudaStream_t stream);
 // local link updates of every chain (closed: no permutation is in use)

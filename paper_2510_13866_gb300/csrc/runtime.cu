@@ -10,6 +10,7 @@
 
 #include "../../include/hqmc.h"
 #include "internal.h"
+#include "window_rule.h"
 
 namespace hqmc {
 cudaError_t launch_ffbs_f32(int L, const DevState &st, const FfbsLaunch &fl, int grid, int wpc, cudaStream_t s);
@@ -253,32 +254,17 @@ void build_tab(const HostChain &h, ChainTab &tb, double lam) {
     for (int m = -kPTab; m <= kPTab; ++m) tb.pplus[m + kPTab] = 1.0 / (1.0 + std::exp(-2.0 * lam * m));
 }
 
+void set_window(const ChainTab &tb, ChainDev &d) {
+    const WinRule w = window_rule(tb.g_d, d.L, std::exp(d.lam));
+    d.win_R = w.R;
+    d.win_min = w.least;
+}
+
 double hirsch_lambda(double U, double dtau) { return std::acosh(std::exp(0.5 * dtau * U)); }
 
 }  // namespace
 
 namespace hqmc {
-// Window of the backward draw (ffbs_window.cuh).  WinR is the least R with g(R + 1) <= 2^-60 g(0):
-// the sites beyond it then hold less than 2^-36 of any total S >= win_min = 2^36 4 g(R + 1) g(0)
-// max W, and win_min stays below 2^-22 of the largest weight, so that almost every draw is
-// answered (t dtau = 1/32, 0.05, 0.1: R = 8, 9, 10).  Hops that need R > kWinHalf - 1 (t dtau
-// above 0.14) leave no margin for the moves between load and draw: no window.
-void window_rule(const ChainTab &tb, int L, double wmax, ChainDev &d) {
-    d.win_R = 0;
-    d.win_min = 0.f;
-    if (L <= 2 * kWinHalf + 1) return;
-    double far = 0.0;  // the largest g beyond R
-    for (int R = L / 2 - 1; R >= 1; --R) {
-        far = std::max(far, tb.g_d[R + 1]);
-        if (far > 0x1.0p-60 * tb.g_d[0]) return;
-        if (R > kWinHalf - 1) continue;
-        const double m = 0x1.0p+36 * 4.0 * far * tb.g_d[0] * wmax;
-        if (!(m < 1e30)) return;
-        d.win_R = R;
-        d.win_min = float(std::max(m, 1e-30));
-    }
-}
-
 // Tables and lambda of one chain, for entry points that do not own a context.
 void host_chain_table(int L, double t, double U, double dtau, ChainTab &tb, double *lam) {
     HostChain h;
@@ -667,7 +653,7 @@ int prepare(hqmc_ctx *c) {
     std::vector<ChainTab> tabs(c->nchains);
     for (int i = 0; i < c->nchains; ++i) {
         build_tab(c->ch[i], tabs[i], c->cdev[i].lam);
-        window_rule(tabs[i], c->ch[i].L, std::exp(c->cdev[i].lam), c->cdev[i]);
+        set_window(tabs[i], c->cdev[i]);
     }
     HQMC_CUDA(c, cudaMemcpyAsync((void *)s.chains, c->cdev.data(), sizeof(ChainDev) * c->nchains, cudaMemcpyHostToDevice, st));
     HQMC_CUDA(c, cudaMemcpyAsync((void *)s.tabs, tabs.data(), sizeof(ChainTab) * c->nchains, cudaMemcpyHostToDevice, st));
@@ -1023,7 +1009,7 @@ int hqmc_set_params(hqmc_ctx *c, int chain, double t, double U, double beta, dou
             d.gcoup = std::sqrt(std::fabs(c->ch[i].U) * c->ch[i].dtau);
             ChainTab tb;
             build_tab(c->ch[i], tb, d.lam);
-            window_rule(tb, c->ch[i].L, std::exp(d.lam), d);
+            set_window(tb, d);
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.chains + i), &d, sizeof(ChainDev), cudaMemcpyHostToDevice, c->stream));
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.tabs + i), &tb, sizeof(ChainTab), cudaMemcpyHostToDevice, c->stream));
             if (d.gauss) {
