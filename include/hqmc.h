@@ -202,9 +202,10 @@ int hqmc_get_class_launch(hqmc_ctx *ctx, int L, int *warps_per_cta);
 int hqmc_autotune(hqmc_ctx *ctx, int trial_sweeps, int *n_tuned);
 
 /* Device memory the context needs (state + scratch), in bytes, for the current
- * parameters and launch configuration.  FP32 contexts with L > 32 that stream f get up to
- * four scratch slots per CTA while the device has the memory for them; a workspace of the
- * size without those extra slots is accepted too.  Errors: HQMC_ERR_STATE before set_params. */
+ * parameters and launch configuration.  FP32 contexts with L > 32 and U >= 0 that stream f
+ * get up to four scratch slots per CTA where hops are short (t dtau up to 0.165) and the extra
+ * slots take at most a quarter of the device memory that is free beyond the rest; a workspace
+ * of the size without them is accepted too.  Errors: HQMC_ERR_STATE before set_params. */
 int hqmc_workspace_size(hqmc_ctx *ctx, size_t *bytes);
 
 /* Hand the context a caller-owned device buffer of at least hqmc_workspace_size bytes,

@@ -64,6 +64,9 @@ struct HostChain {
 
 // Scratch of a wide FP32 class up to which its CTAs take several slots each: 5% of the device
 constexpr size_t kBatchBytes = size_t(14) << 30;
+// and the share of the device's free memory, after the layout without them, that the extra slots
+// may take: the rest is for the adjoint's scratch and the caller's own tensors
+constexpr size_t kBatchShare = 4;
 
 // Read-backs up to this size go through a context's pinned staging buffer.
 constexpr size_t kPinBytes = size_t(256) << 10;
@@ -154,6 +157,7 @@ struct hqmc_ctx {
     bool keep_started = false;
 
     bool batch_units = true;  // several slots per CTA of the wide classes (off where memory is short)
+    size_t batch_extra = 0;   // bytes of the layout that are slots beyond the first
 
     // adjoint: checkpoint stride (0 = ceil(sqrt M)) and format, context-owned scratch
     int ckpt_stride = 0;
@@ -254,13 +258,13 @@ void build_tab(const HostChain &h, ChainTab &tb, double lam) {
     for (int m = -kPTab; m <= kPTab; ++m) tb.pplus[m + kPTab] = 1.0 / (1.0 + std::exp(-2.0 * lam * m));
 }
 
+double hirsch_lambda(double U, double dtau) { return std::acosh(std::exp(0.5 * dtau * U)); }
+
 void set_window(const ChainTab &tb, ChainDev &d) {
     const WinRule w = window_rule(tb.g_d, d.L, std::exp(d.lam));
     d.win_R = w.R;
     d.win_min = w.least;
 }
-
-double hirsch_lambda(double U, double dtau) { return std::acosh(std::exp(0.5 * dtau * U)); }
 
 }  // namespace
 
@@ -357,6 +361,20 @@ int default_wpc(hqmc_ctx *c, int L) {
     return w;
 }
 
+// A wide class draws some chain's worldlines from windows: no Gaussian field in it (those run another
+// instantiation), and short enough hops (window_rule).
+bool draws_windows(const hqmc_ctx *c, const LClass &k) {
+    for (int i : k.chains)
+        if (c->ch[i].U < 0.0) return false;
+    std::vector<double> g;
+    for (int i : k.chains) {
+        const HostChain &h = c->ch[i];
+        ring_propagator(h.L, h.t * h.dtau, g);
+        if (window_rule(g.data(), h.L, std::exp(hirsch_lambda(h.U, h.dtau))).R > 0) return true;
+    }
+    return false;
+}
+
 // Compute the device layout (offsets) and its size; fills c->classes, c->cdev.
 int plan_layout(hqmc_ctx *c, size_t *total) {
     const int nc = c->nchains;
@@ -364,6 +382,7 @@ int plan_layout(hqmc_ctx *c, size_t *total) {
         if (!c->ch[i].set) return fail(c, HQMC_ERR_STATE, "set_params has not been called for every chain");
     const bool f64 = c->precision == HQMC_FP64;
     c->cdev.assign(nc, ChainDev{});
+    c->batch_extra = 0;
     // classes by L
     c->classes.clear();
     for (int i = 0; i < nc; ++i) {
@@ -524,12 +543,14 @@ int plan_layout(hqmc_ctx *c, size_t *total) {
         k.slot_elems = (per_wl + aux) * (is_big(k.L) ? ffbs_wide_wpc(k.L) : 1);
         const size_t elem = is_big(k.L) ? (f64 ? 8 : 4) : (f64 ? 16 : 8);
         k.scratch_bytes = size_t(k.groups) * size_t(k.slot_elems) * elem;
-        // wide FP32 classes that stream f: more slots per CTA, so that several units are drawn
-        // at once, while the class stays within kBatchBytes and every CTA has the units
+        // wide FP32 Hirsch classes that stream f and draw from windows: more slots per CTA, so that
+        // several units are drawn at once, while the class stays within kBatchBytes and every CTA
+        // has the units.  Whole slices are drawn unit by unit and need one slot.
         k.batch = 1;
-        if (is_big(k.L) && !f64 && k.ckpt_K == 0 && c->batch_units) {
+        if (is_big(k.L) && !f64 && k.ckpt_K == 0 && c->batch_units && draws_windows(c, k)) {
             const long long most = std::min<long long>(kBatchBytes / k.scratch_bytes, (k.total_units + k.grid - 1) / k.grid);
             k.batch = int(std::max(1LL, std::min<long long>(ffbs_wide_batch(k.L), most)));
+            c->batch_extra += k.scratch_bytes * (k.batch - 1);
             k.scratch_bytes *= k.batch;
         }
         k.scratch_off = take(k.scratch_bytes);
@@ -576,6 +597,19 @@ int plan_within(hqmc_ctx *c, size_t limit, size_t *need) {
     return plan_layout(c, need);
 }
 
+// plan_layout for memory that is still to be allocated: with the extra slots where they take at most
+// 1 / kBatchShare of what the device has free beyond the rest (or what is attached holds them).
+int plan_free(hqmc_ctx *c, size_t *need) {
+    int rc = plan_within(c, SIZE_MAX, need);
+    if (rc || c->batch_extra == 0 || *need <= c->attached_bytes) return rc;
+    size_t room = 0, total = 0;
+    HQMC_CUDA(c, cudaSetDevice(c->device));
+    HQMC_CUDA(c, cudaMemGetInfo(&room, &total));
+    const size_t rest = *need - c->batch_extra;
+    if (room > rest && c->batch_extra <= (room - rest) / kBatchShare) return rc;
+    return plan_within(c, 0, need);
+}
+
 // What is queued on the legacy default stream so far comes before what the context enqueues from here on.
 // A context whose stream was given as NULL runs on a non-blocking stream of its own, which does not wait for the
 // default stream by itself; the device memory that a caller hands over (a workspace, v, dlogZ_dv) may still be
@@ -593,7 +627,7 @@ int prepare(hqmc_ctx *c) {
     if (c->ready) return HQMC_OK;
     HQMC_CUDA(c, cudaSetDevice(c->device));
     size_t need = 0;
-    int rc = plan_within(c, c->attached ? c->attached_bytes : SIZE_MAX, &need);
+    int rc = c->attached ? plan_within(c, c->attached_bytes, &need) : plan_free(c, &need);
     if (rc) return rc;
     if (c->attached) {
         if (c->attached_bytes < need) return fail(c, HQMC_ERR_NOMEM, "attached workspace too small");
@@ -1267,17 +1301,7 @@ int hqmc_workspace_size(hqmc_ctx *c, size_t *bytes) {
     auto keep_cdev = c->cdev;
     auto keep_cls = c->classes;
     const bool keep_batch = c->batch_units;
-    int rc = plan_within(c, SIZE_MAX, &need);
-    bool extra = false;
-    for (auto &k : c->classes) extra = extra || k.batch > 1;
-    if (!rc && extra) {
-        // the wide classes' extra slots are asked for only where the device has the room for them (or
-        // what is attached already holds them)
-        size_t room = 0, total = 0;
-        HQMC_CUDA(c, cudaSetDevice(c->device));
-        HQMC_CUDA(c, cudaMemGetInfo(&room, &total));
-        rc = plan_within(c, std::max(room, c->attached_bytes), &need);
-    }
+    int rc = plan_free(c, &need);
     if (c->ready) {
         c->st = keep;
         c->cdev = keep_cdev;
