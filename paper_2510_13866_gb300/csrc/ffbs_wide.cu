@@ -1,5 +1,7 @@
 // ffbs_wide.cu -- instantiations of the wide-lattice FFBS kernel (L = 48, 64, 128; FP32
 // and FP64) for Hirsch-field classes, and the host-side geometry.
+#include <algorithm>
+
 #include "ffbs_launch.cuh"
 #include "ffbs_wide.cuh"
 
@@ -7,6 +9,8 @@ namespace hqmc {
 
 cudaError_t ffbs_wide_occupancy_g(int L, bool fp64, int *blocks);
 cudaError_t launch_ffbs_wide_g(int L, bool fp64, const DevState &st, const FfbsLaunch &fl, int grid, cudaStream_t s);
+cudaError_t ffbs_wide_occupancy_w(int L, int *blocks);
+cudaError_t launch_ffbs_wide_w(int L, const DevState &st, const FfbsLaunch &fl, int grid, cudaStream_t s);
 
 bool ffbs_wide_supported(int L) {
     switch (L) {
@@ -29,29 +33,23 @@ int ffbs_wide_wpc(int L) {
     }
 }
 
-// units that a CTA of the FP32 streaming kernel filters before it draws their worldlines
-int ffbs_wide_batch(int L) {
-    switch (L) {
-#define HQMC_CASE(n) \
-    case n: return WideGeo<float, n>::NB;
-        HQMC_WIDE_SIZES(HQMC_CASE)
-#undef HQMC_CASE
-        default: return 1;
-    }
-}
-
-// both Gaussian flags get their limits; the grid follows the smaller residency
+// every instantiation gets its limit; the grid follows the smallest residency
 cudaError_t ffbs_wide_occupancy(int L, bool fp64, int *blocks) {
     cudaError_t e = wide_occ_dispatch<false>(L, fp64, blocks);
     if (e != cudaSuccess) return e;
-    int bg = 0;
-    e = ffbs_wide_occupancy_g(L, fp64, &bg);
-    if (e == cudaSuccess && bg > 0 && bg < *blocks) *blocks = bg;
+    int other = 0;
+    e = ffbs_wide_occupancy_g(L, fp64, &other);
+    if (e == cudaSuccess && other > 0) *blocks = std::min(*blocks, other);
+    if (e != cudaSuccess || fp64) return e;
+    e = ffbs_wide_occupancy_w(L, &other);
+    if (e == cudaSuccess && other > 0) *blocks = std::min(*blocks, other);
     return e;
 }
 
 cudaError_t launch_ffbs_wide(int L, bool fp64, const DevState &st, const FfbsLaunch &fl, int grid, cudaStream_t s) {
-    return fl.gauss ? launch_ffbs_wide_g(L, fp64, st, fl, grid, s) : wide_launch_dispatch<false>(L, fp64, st, fl, grid, s);
+    if (fl.gauss) return launch_ffbs_wide_g(L, fp64, st, fl, grid, s);
+    if (!fp64 && fl.ckpt_K == 0 && fl.windows) return launch_ffbs_wide_w(L, st, fl, grid, s);
+    return wide_launch_dispatch<false>(L, fp64, st, fl, grid, s);
 }
 
 }  // namespace hqmc

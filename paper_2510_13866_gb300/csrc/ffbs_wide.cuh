@@ -40,7 +40,11 @@ namespace hqmc {
 template <int L>
 constexpr int kWideBatch = L == 48 ? 3 : L / 32;
 
-template <typename T, int L>
+// Shared memory of a CTA.  WIN: the instantiation that draws from windows; the others and the adjoint
+// do without its rings and per-unit copies, which leave less of the SM's memory as L1 (L = 64: 25.4
+// against 18.3 KB for each of eight CTAs; with the larger size everywhere a Gaussian class of L = 48
+// took 10.37 instead of 9.80 ms a sweep, the adjoint of L = 64 3.40 instead of 3.34).
+template <typename T, int L, bool WIN = false>
 struct WideGeo {
     static constexpr int WPC = (L % 32 == 0) ? 1 : 2;  // worldlines per CTA
     static constexpr int NT = WPC * L;                    // threads: one per (worldline, line)
@@ -54,13 +58,13 @@ struct WideGeo {
     static constexpr size_t XB = a16(XTR > XPF ? XTR : XPF);
     // FP32 streaming: units whose worldlines are drawn together after their forward passes
     // (kWideBatch), and one window ring per warp in the place of the transpose buffers
-    static constexpr int NB = sizeof(T) == 4 ? kWideBatch<L> : 1;
-    static constexpr size_t XALL = sizeof(T) == 4 && NW * kWinBytes > WPC * XB ? NW * kWinBytes : WPC * XB;
+    static constexpr int NB = WIN ? kWideBatch<L> : 1;
+    static constexpr size_t XALL = WIN && NW * kWinBytes > WPC * XB ? NW * kWinBytes : WPC * XB;
     static constexpr size_t MIXB = a16(size_t(2 * L) * sizeof(T));  // (al, -al, be, -be) per k
     static constexpr size_t G2B = a16(size_t(2 * L) * sizeof(T));  // per unit of a batch
     static constexpr size_t WXB = a16(size_t(WPC) * L * sizeof(T));
     static constexpr size_t HLB = a16(size_t(L) * sizeof(float));  // per unit of a batch
-    static constexpr size_t UNB = a16(NB * sizeof(WinUnit));
+    static constexpr size_t UNB = WIN ? a16(NB * sizeof(WinUnit)) : 0;
     static constexpr size_t REDB = a16(size_t(2 * NW * WPC + 4 * WPC) * sizeof(T));
     static constexpr size_t IB = 64;  // work unit, crossings, fallbacks, end exponents
     static constexpr size_t UB = a16(size_t(WPC) * 8);
@@ -172,10 +176,13 @@ __device__ __forceinline__ T wl_warp_max(T v) {
 // (FP32 only); the streaming instantiation carries none of that code.  GAUSS: the class
 // holds Gaussian-field chains (U < 0), whose potentials are read from the sigma field's
 // tables and whose log-weight estimate is summed in the backward pass; the Hirsch-only
-// instantiation carries none of that code.
-template <typename T, int L, bool CKPT, bool GAUSS>
+// instantiation carries none of that code.  WIN: some chain of the class draws from windows (FP32,
+// streamed, Hirsch fields); a class of longer hops runs without them (L = 48, t dtau = 0.2: 5.57
+// instead of 5.75 ms, the window draw costs the whole-slice draw registers).
+template <typename T, int L, bool CKPT, bool GAUSS, bool WIN>
 __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_wide_kernel(DevState st, FfbsLaunch fl) {
-    using G = WideGeo<T, L>;
+    static_assert(!WIN || (sizeof(T) == 4 && !CKPT && !GAUSS), "window draws");
+    using G = WideGeo<T, L, WIN>;
     constexpr int WPC = G::WPC, NT = G::NT, NW = G::NW, CH = G::CH, LP = G::LP, N = L * L;
     constexpr int NCH = N / CH;  // 16-byte chunks per slice of one worldline
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -206,7 +213,6 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
     T *xb = reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(xbuf_all) + w * G::XB);
     T *wx = wx_all + w * L;
     const uint64_t sweep = *st.sweep;
-    constexpr bool WIN = sizeof(T) == 4 && !CKPT && !GAUSS;
     // fl.batch slots per CTA: one for each unit that waits to be drawn
     T *slot0 = reinterpret_cast<T *>(fl.scratch) + (long long)blockIdx.x * fl.batch * fl.slot_elems;
     int nwait = 0;
@@ -732,44 +738,46 @@ __global__ void __launch_bounds__(WideGeo<T, L>::NT, WideGeo<T, L>::MINB) ffbs_w
 
 #define HQMC_WIDE_SIZES(X) X(48) X(64) X(128)
 
-// host side, per Gaussian flag: raise the kernels' shared-memory limits and return the
-// residency of the streaming instantiation; launch the class's instantiation (the limit is
-// raised beforehand, never during stream capture)
-template <typename T, int L, bool G>
+// host side, per instantiation: raise its shared-memory limit (beforehand, never during stream
+// capture) and return its residency; launch it
+template <typename T, int L, bool CKPT, bool GAUSS, bool WIN>
 cudaError_t wide_occ(int *blocks) {
-    if constexpr (sizeof(T) == 4) {
-        cudaError_t e = raise_smem_limit(ffbs_wide_kernel<T, L, true, G>, WideGeo<T, L>::BYTES);
-        if (e != cudaSuccess) return e;
-    }
-    auto k = ffbs_wide_kernel<T, L, false, G>;
-    cudaError_t e = raise_smem_limit(k, WideGeo<T, L>::BYTES);
+    auto k = ffbs_wide_kernel<T, L, CKPT, GAUSS, WIN>;
+    cudaError_t e = raise_smem_limit(k, WideGeo<T, L, WIN>::BYTES);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, WideGeo<T, L>::NT, WideGeo<T, L>::BYTES);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, WideGeo<T, L>::NT, WideGeo<T, L, WIN>::BYTES);
 }
 
+template <typename T, int L, bool CKPT, bool GAUSS, bool WIN>
+cudaError_t wide_go(const DevState &st, const FfbsLaunch &fl, int grid, cudaStream_t s) {
+    ffbs_wide_kernel<T, L, CKPT, GAUSS, WIN><<<grid, WideGeo<T, L>::NT, WideGeo<T, L, WIN>::BYTES, s>>>(st, fl);
+    return cudaGetLastError();
+}
+
+// the instantiations without windows: the residency is the streaming one's
 template <bool G>
 cudaError_t wide_occ_dispatch(int L, bool fp64, int *blocks) {
+    cudaError_t e = cudaErrorInvalidValue;
     switch (L) {
-#define HQMC_CASE(n) \
-    case n: return fp64 ? wide_occ<double, n, G>(blocks) : wide_occ<float, n, G>(blocks);
+#define HQMC_CASE(n)                                                       \
+    case n:                                                                \
+        if (fp64) return wide_occ<double, n, false, G, false>(blocks);     \
+        e = wide_occ<float, n, true, G, false>(blocks);                    \
+        return e != cudaSuccess ? e : wide_occ<float, n, false, G, false>(blocks);
         HQMC_WIDE_SIZES(HQMC_CASE)
 #undef HQMC_CASE
-        default: return cudaErrorInvalidValue;
+        default: return e;
     }
 }
 
 template <bool G>
 cudaError_t wide_launch_dispatch(int L, bool fp64, const DevState &st, const FfbsLaunch &fl, int grid, cudaStream_t s) {
     switch (L) {
-#define HQMC_CASE(n)                                                                                           \
-    case n:                                                                                                    \
-        if (fp64)                                                                                              \
-            ffbs_wide_kernel<double, n, false, G><<<grid, WideGeo<double, n>::NT, WideGeo<double, n>::BYTES, s>>>(st, fl); \
-        else if (fl.ckpt_K > 0)                                                                               \
-            ffbs_wide_kernel<float, n, true, G><<<grid, WideGeo<float, n>::NT, WideGeo<float, n>::BYTES, s>>>(st, fl);     \
-        else                                                                                                   \
-            ffbs_wide_kernel<float, n, false, G><<<grid, WideGeo<float, n>::NT, WideGeo<float, n>::BYTES, s>>>(st, fl);    \
-        return cudaGetLastError();
+#define HQMC_CASE(n)                                                              \
+    case n:                                                                       \
+        if (fp64) return wide_go<double, n, false, G, false>(st, fl, grid, s);    \
+        if (fl.ckpt_K > 0) return wide_go<float, n, true, G, false>(st, fl, grid, s); \
+        return wide_go<float, n, false, G, false>(st, fl, grid, s);
         HQMC_WIDE_SIZES(HQMC_CASE)
 #undef HQMC_CASE
         default: return cudaErrorInvalidValue;

@@ -136,6 +136,7 @@ struct FfbsLaunch {
     int ckpt_bf16;
     long long seg_off;
     int gauss;                 // some chain of the class has a Gaussian field (U < 0)
+    int windows;               // some chain of the class draws from windows (wide kernel)
     int batch;                 // wide kernel: slots per CTA (units filtered before they are drawn)
 };
 

@@ -848,7 +848,10 @@ int enqueue_sweep(hqmc_ctx *c, cudaStream_t st, bool capture) {
         HQMC_CUDA(c, cudaMemsetAsync(fl.next_unit, 0, sizeof(unsigned), s));
         const int wpc = default_wpc(c, cl.L);
         fl.gauss = 0;
-        for (int ci : cl.chains) fl.gauss |= c->cdev[ci].gauss;
+        for (int ci : cl.chains) {
+            fl.gauss |= c->cdev[ci].gauss;
+            fl.windows |= c->cdev[ci].win_R > 0;
+        }
         cudaError_t e = is_big(cl.L) ? launch_ffbs_wide(cl.L, f64, c->st, fl, cl.grid, s)
                         : f64 ? (fl.gauss ? launch_ffbs_f64g(cl.L, c->st, fl, cl.grid, wpc, s)
                                           : launch_ffbs_f64(cl.L, c->st, fl, cl.grid, wpc, s))
@@ -1043,7 +1046,9 @@ int hqmc_set_params(hqmc_ctx *c, int chain, double t, double U, double beta, dou
             d.gcoup = std::sqrt(std::fabs(c->ch[i].U) * c->ch[i].dtau);
             ChainTab tb;
             build_tab(c->ch[i], tb, d.lam);
+            const int win_R = d.win_R;
             set_window(tb, d);
+            if ((d.win_R > 0) != (win_R > 0)) drop_graph(c);  // it holds the class's instantiation
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.chains + i), &d, sizeof(ChainDev), cudaMemcpyHostToDevice, c->stream));
             HQMC_CUDA(c, cudaMemcpyAsync((void *)(c->st.tabs + i), &tb, sizeof(ChainTab), cudaMemcpyHostToDevice, c->stream));
             if (d.gauss) {
