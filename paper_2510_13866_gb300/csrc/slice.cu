@@ -6,6 +6,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "slice_math.h"
 
 namespace hqmc {
 
@@ -35,20 +36,6 @@ struct SliceSmem {
 };
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
-
-// Integer threshold of a Gibbs draw: with u = k 2^-53 (k the word's leading 53 bits),
-// u < p if and only if k < ceil(p 2^53); p 2^53 is exact.  The draws then take no FP64 operation per
-// site (two per cycle and SM).  With div_n and the unrolled transforms below the kernel takes 161
-// instead of 177 us for 64 chains of L = 32 (M = 80), the grouped form 37.5 instead of 43.5 us for
-// 32 of L = 12 (M = 120).
-__device__ __forceinline__ unsigned long long gibbs_threshold(double p) { return (unsigned long long)ceil(p * 0x1.0p53); }
-
-// x / N for an integer N < 2^15 with inv = 1 / N correctly rounded: the correctly rounded quotient by
-// one residual (Markstein, IBM J. Res. Dev. 34, 1990), exact in one product when N is a power of two.
-__device__ __forceinline__ double div_n(double x, double n, double inv, bool pow2) {
-    const double q = x * inv;
-    return pow2 ? q : fma(fma(-q, n, x), inv, q);
-}
 
 // One term of the direct transform of a line: z += a w, for a real a and for a complex one (the
 // order of the roundings is spelled out: it is part of S(k)'s last bits).
