@@ -167,8 +167,9 @@ int hqmc_set_stream(hqmc_ctx *ctx, void *stream);
 /* Launch configuration: use_graph = replay one captured CUDA graph per sweep;
  * persistent = size the FFBS grid to the resident capacity (each worldline group
  * loops over pairs) instead of one group per pair; warps_per_cta in {1,2,4,8}
- * (0 = default: 4, or fewer in an FP64 context too small to fill the SMs with 4).  Takes effect at the next sweep; a change of grid or shape re-lays
- * the context out as described at hqmc_set_class_launch.  Errors: HQMC_ERR_ARG. */
+ * (0 = default: 4, or fewer in an FP64 context too small to fill the SMs with 4).  Takes
+ * effect at the next sweep; a change of grid or shape re-lays the context out as described at
+ * hqmc_set_class_launch.  Errors: HQMC_ERR_ARG. */
 int hqmc_set_launch(hqmc_ctx *ctx, int use_graph, int persistent, int warps_per_cta);
 
 /* Slices of one chain handled by one CTA of the Gibbs/measure kernel.  Up to L = 12 (the

@@ -8,15 +8,16 @@
 // 33% with L = 48).  Here a warp reads (2H+1) lines x 28 elements around x_{i+1} (2.7 KB
 // instead of 16 KB at L = 64, 64 KB at L = 128) and draws from them alone.
 //
-// The draw is the same draw.  Sites beyond WinR steps hold at most
+// The draw is the same but for 2^-36 of its probability.  Sites beyond WinR steps hold at most
 //     g(WinR + 1) g(0) sum_y f(y) <= 4 g(WinR + 1) g(0) max W
 // of the conditional's total S (the message is normalised to a sum in [1, 2)); the window
-// answers only where that is below 2^-36 S (S >= win_min, a per-chain constant), 4096 times
-// below the rounding of S itself.  Inside the window the arithmetic is the whole row's:
-// the same in-row prefix in the order of x, and row totals scanned in the association of the
-// whole-slice form (rows outside the window enter as zeros).  Where a vanishing weight could
-// still decide -- a uniform of 0, a target equal to a row boundary, no crossing -- the warp
-// draws from the whole slice (draw_whole), row by row.
+// answers only where that is below 2^-36 S (S >= win_min, a per-chain constant): 4096 times
+// below the rounding of S itself and of the 24-bit uniform, though a target near the start of the
+// CDF is compared at a finer spacing than that, and such a draw may differ.  Inside the window the
+// arithmetic is the whole row's: the same in-row prefix in the order of x, and row totals scanned
+// in the association of the whole-slice form (rows outside the window enter as zeros), so all other
+// draws are equal.  Where a vanishing weight could still decide -- a uniform of 0, a target equal to
+// a row boundary, no crossing -- the warp draws from the whole slice (draw_whole), row by row.
 //
 // Loads run kWinStages slices ahead, centred on the worldline's site at that time; the margin
 // kWinH - WinR covers the steps in between, and a worldline that left it (4 steps one way in

@@ -28,7 +28,9 @@
 // segment before it then recomputes one step further.
 // Carrying (dG/dt) * b as a second message took 7 half-length FFTs and two transposes per reverse
 // slice instead of 4 and one.  The kernel is bound by the FMA pipe: L = 16, M = 80, 128 chains with a
-// given v, 2.87 ms before this and exp_table_kernel, 2.17 ms with both (and 35 us for the table).
+// given v, 2.87 ms before this and exp_table_kernel, 2.17 ms with both (and 35 us for the table); the
+// rare longer segment adds 1% to a step (2.745 -> 2.775 ms; with a convolution of its own after the
+// loop 2.755, but 13.0 instead of 8.5 KB of spill in FP64 at L = 32).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
     using FG = FfbsGeo<T, L>;
     using V = vec2_t<T>;
     constexpr int N = L * L;
-    constexpr int GW = FG::GW, LP = FG::LP, CH = FG::CH;
+    constexpr int GW = FG::GW, LP = FG::LP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -84,7 +86,6 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
     V *xbuf = reinterpret_cast<V *>(gsm);
     V *mixg = reinterpret_cast<V *>(gsm + G::XBUF);
     const long long gid = ((long long)blockIdx.x * wpc + warp) * FG::GPW + gw;
-    const long long ngroups = (long long)gridDim.x * wpc * FG::GPW;
     unsigned char *ck = reinterpret_cast<unsigned char *>(gk.ckpt) + gid * gk.ckpt_bytes;
     V *seg = reinterpret_cast<V *>(gk.seg) + gid * gk.seg_elems;
     const T *vlog_all = reinterpret_cast<const T *>(gk.v);
@@ -106,7 +107,6 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         }
     };
 
-    (void)ngroups;
     for (;;) {
         unsigned qn = 0;
         if (gl == 0) qn = atomicAdd(gk.next_pair, 1u);
@@ -458,7 +458,6 @@ __global__ void __launch_bounds__(128) grad_kernel(DevState st, GradLaunch gk) {
         if (gl == 0) atomicAdd(&gk.dt[c], cd.beta / M * (double(dts0) + (has1 ? double(dts1) : 0.0)));
         __syncwarp(gmask);
     }
-    (void)CH;
 }
 
 template <typename T, int L>

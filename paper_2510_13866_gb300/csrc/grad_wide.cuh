@@ -25,8 +25,8 @@ namespace hqmc {
 
 // Resident CTAs per SM the adjoint's registers are sized for: as the FFBS kernel's, but four at L = 48
 // in FP32 (168 registers without spills; at six, 96 registers and 888 bytes of spill, 2 chains of
-// M = 40 and 300 worldlines per spin took 1.62 ms instead of 1.41).  At L = 64 the spills of eight
-// CTAs (128 registers) cost less than four CTAs' lost warps (3.37 against 3.73 ms at 512 worldlines).
+// M = 40 and 300 worldlines per spin take 1.51 ms instead of 1.40).  At L = 64 the spills of eight
+// CTAs (128 registers) cost less than four CTAs' lost warps (3.43 against 3.72 ms at 512 worldlines).
 template <typename T, int L>
 constexpr int kGradMinBlocks = (sizeof(T) == 4 && L == 48) ? 4 : WideGeo<T, L>::MINB;
 
